@@ -719,7 +719,8 @@ extern "C" int lsnif_load_object(lsnif_ctx *ctx, const lsnif_object_desc *desc, 
   d.umma_lo_bytes = (uint32_t)(((wbytes - (size_t)cfg.width * d.n_in * 2) + 15) & ~size_t(15));
   OALLOC(umma_lo, const uint8_t *, d.umma_lo_bytes, "BF16 residual weights");
   OALLOC(w0_16c, const uint8_t *, (size_t)cfg.width * d.n_in * 2, "chunk-major FP16 first layer");
-  OALLOC(plain_out, const float *, 4 * ((size_t)d.n_out_pad * cfg.width + d.n_out_pad), "padded output layer");
+  OALLOC(plain_out, const float *, 4 * ((size_t)d.n_out_pad * cfg.width + d.n_out_pad + kNonFiniteWords),
+         "padded output layer");
   cudaError_t e = cudaMemcpy((void *)d.occ, occ.data(), 4 * occ.size(), cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaMemcpy((void *)d.dist, dist.data(), dist.size(), cudaMemcpyHostToDevice);
   if (e != cudaSuccess) { free_object(ctx, o); return cuda_fail(e, "upload occupancy"); }

@@ -18,6 +18,7 @@ constexpr int kMaxCap = 32;          // H/2 <= 32
 constexpr int kBuckets = kMaxCap + 1;  // per object: k = 0..32
 constexpr int kTileM = 128;          // rays per tensor-core tile (tcgen05 M)
 constexpr int kDistCap = 32;         // largest stored occupancy distance
+constexpr int kNonFiniteWords = 16;  // per object: words that are nonzero when a first-layer weight is not finite
 
 inline bool valid_precision(int p) {
   return p == LSNIF_FP32_PLAIN || p == LSNIF_BF16_FUSED || p == LSNIF_FP8_FUSED || p == LSNIF_FP16_FUSED;
@@ -73,7 +74,7 @@ struct DevObject {
   // chunk s (network inputs [s CHK, (s+1) CHK), CHK = 2 L F: two points) is a
   // contiguous W x CHK core-matrix slice, so one bulk copy moves it
   const uint8_t *w0_16c;
-  const float *plain_out;  // FP32 output layer padded to n_out_pad rows, then its bias
+  const float *plain_out;  // FP32 output layer padded to n_out_pad rows, its bias, then kNonFiniteWords int32
 
   // kept mesh (training labels): per-voxel triangle lists in CSR form
   const float *verts;
@@ -175,6 +176,10 @@ cudaError_t launch_group(const QueryLaunch &q, int *launches);
 // entries and receives the total at sums[(n + 1023) / 1024]
 cudaError_t launch_exclusive_scan(int32_t *v, int64_t n, int32_t *sums, cudaStream_t st);
 cudaError_t launch_plain_tail(const QueryLaunch &q, int ldx, int chunk_tiles, int *launches);
+// one kernel for gather, network and decode where every object has this F
+// and width; lf_max: the largest L F among them (plain.cu)
+bool plain_fused_supported(int F, int width, int lf_max);
+cudaError_t launch_plain_fused(const QueryLaunch &q, int F, int width, int lf_max, int *launches);
 cudaError_t launch_trace_only(const DevObject *dobj, const RaysArg &rays, int32_t *k, float *t01,
                               float *pts, int32_t *vox, int *err, cudaStream_t st);
 cudaError_t launch_encode(const DevObject *dobj, const DevObject &host_obj, const float *pts, int64_t n,

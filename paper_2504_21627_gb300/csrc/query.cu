@@ -1257,8 +1257,15 @@ __global__ void build_umma_kernel(DevObject h, uint8_t *dst, uint8_t *dst16, uin
   }
 }
 
-// FP32 output layer padded with zero rows to n_out_pad (plain SIMT path).
-__global__ void build_plain_out_kernel(DevObject h, float *dst) {
+// FP32 output layer padded with zero rows to n_out_pad (FP32 path), and, one
+// word per block, whether this block saw a first-layer weight that is not
+// finite (kNonFiniteWords blocks).
+__global__ void __launch_bounds__(256) build_plain_out_kernel(DevObject h, float *dst) {
+  bool bad = false;
+  for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < h.width * h.n_in; i += gridDim.x * blockDim.x)
+    bad |= !isfinite(h.mlp32[i]);
+  const int any = __syncthreads_or(bad);
+  if (threadIdx.x == 0) reinterpret_cast<int *>(dst + (size_t)h.n_out_pad * (h.width + 1))[blockIdx.x] = any;
   const float *p = h.mlp32;
   int fan_in = h.n_in;
   for (int l = 0; l < h.n_hidden; ++l) {
@@ -1281,7 +1288,7 @@ __global__ void build_plain_out_kernel(DevObject h, float *dst) {
 cudaError_t launch_build_umma(const DevObject &h, cudaStream_t st) {
   build_umma_kernel<<<152, 256, 0, st>>>(h, const_cast<uint8_t *>(h.umma), const_cast<uint8_t *>(h.umma_h),
                                          const_cast<uint8_t *>(h.umma_lo), const_cast<uint8_t *>(h.w0_16c));
-  build_plain_out_kernel<<<16, 256, 0, st>>>(h, const_cast<float *>(h.plain_out));
+  build_plain_out_kernel<<<kNonFiniteWords, 256, 0, st>>>(h, const_cast<float *>(h.plain_out));
   return cudaGetLastError();
 }
 

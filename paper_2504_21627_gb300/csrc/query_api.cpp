@@ -108,6 +108,13 @@ struct Shape {
   uint32_t umma_max = 0, umma_lo_max = 0;
   bool mixed_fused = false;      // objects differ in F or width
   bool has_mesh = false;         // some object of the batch is a mesh object
+  int lf_max = 0;                // largest L F
+  bool one_plain = true;         // every object has the representative's F and width
+
+  // FP32: one fused kernel, or features materialised for the stage kernels
+  bool plain_fused() const { return rep && one_plain && plain_fused_supported(rep->d.F, rep->d.width, lf_max); }
+  // columns of the FP32 feature scratch a query of this precision needs
+  int feature_cols(int precision) const { return precision == LSNIF_FP32_PLAIN && !plain_fused() ? n_in : 0; }
 };
 
 static int shape_of(lsnif_ctx *ctx, const lsnif_rays *r, Shape *sh) {
@@ -121,6 +128,8 @@ static int shape_of(lsnif_ctx *ctx, const lsnif_rays *r, Shape *sh) {
     sh->wmax = std::max(sh->wmax, std::max(o->d.width, o->d.n_out_pad));
     sh->umma_max = std::max(sh->umma_max, o->d.umma_bytes);
     sh->umma_lo_max = std::max(sh->umma_lo_max, o->d.umma_lo_bytes);
+    sh->lf_max = std::max(sh->lf_max, o->d.L * o->d.F);
+    if (sh->rep && (sh->rep->d.F != o->d.F || sh->rep->d.width != o->d.width)) sh->one_plain = false;
     if (!sh->rep) sh->rep = o;
     else if (sh->rep->d.F != o->d.F || sh->rep->d.width != o->d.width || o->d.L > 16) sh->mixed_fused = true;
   };
@@ -214,7 +223,7 @@ int lsnif::run_query(lsnif_ctx *ctx, Workspace *ws, const lsnif_rays *r, lsnif_h
                                            "and one shape for all objects; BF16 also weights that fit shared memory");
     }
   }
-  const int n_in = precision == LSNIF_FP32_PLAIN ? sh.n_in : 0;
+  const int n_in = sh.feature_cols(precision);
   if ((rc = ensure_workspace(ctx, ws, r->n, sh.H, sh.n_slots, n_in))) return rc;
   QueryLaunch q{};
   q.objs = ctx->d_objs;
@@ -236,7 +245,9 @@ int lsnif::run_query(lsnif_ctx *ctx, Workspace *ws, const lsnif_rays *r, lsnif_h
   if (e == cudaSuccess) e = launch_group(q, &launches);
   if (profile) cudaEventRecord(ctx->ev[2], st);
   if (e == cudaSuccess) {
-    if (precision == LSNIF_FP32_PLAIN) e = launch_plain_tail(q, ws->cap_nin, kChunkTiles, &launches);
+    if (precision == LSNIF_FP32_PLAIN && sh.plain_fused())
+      e = launch_plain_fused(q, rep.F, rep.width, sh.lf_max, &launches);
+    else if (precision == LSNIF_FP32_PLAIN) e = launch_plain_tail(q, ws->cap_nin, kChunkTiles, &launches);
     else if (precision == LSNIF_FP8_FUSED) e = launch_fused8(q, rep, ctx->fp8_variant, &launches);
     else if (streamed) e = launch_fused16s(q, rep, &launches);
     else
@@ -276,7 +287,7 @@ static int query_graph(lsnif_ctx *ctx, const lsnif_rays *r, lsnif_hits *h, int p
   Shape sh;
   if ((rc = shape_of(ctx, r, &sh))) return rc;
   if (!sh.rep) return run_query(ctx, &ctx->ws, r, h, precision, st, false);
-  const int n_in = precision == LSNIF_FP32_PLAIN ? sh.n_in : 0;
+  const int n_in = sh.feature_cols(precision);
   if ((rc = ensure_workspace(ctx, &ctx->ws, r->n, sh.H, sh.n_slots, n_in))) return rc;
   if (ctx->graphs_ws != ctx->ws.base) clear_graphs(ctx);
   std::vector<uint64_t> key = {(uint64_t)r->n, (uint64_t)precision,
