@@ -165,10 +165,14 @@ __global__ void __launch_bounds__(256) presort_scatter_kernel(QueryLaunch q) {
 }
 
 // ---------------------------------------------------------------------------
-// Persistent-lane traversal: after each round of cells a warp hands a new
-// ray to every lane whose ray finished (global ray counter, warp-aggregated).
-// Rays need anywhere from 0 to 3V DDA steps; with one ray per thread a warp
-// runs as long as its longest ray.
+// Persistent-lane traversal: a lane whose ray finished takes another one, so
+// that a warp does not run as long as its longest ray (0 to 3V DDA steps).
+//
+// Starting rays: a warp takes 32 rays at a time from a global counter, all
+// lanes start one each (unit-cube transform, slab test, first voxel -- nine
+// divisions), rays that miss their box are answered at once, and the others
+// go to a queue in shared memory. Idle lanes pop from the queue. The start
+// thus runs with all lanes, which a lane-by-lane refill did not (18 of 32).
 //
 // Empty-space skipping: every iteration crosses one cell: the cube of
 // voxels within Chebyshev distance r of the current voxel, where r + 1 is
@@ -181,63 +185,93 @@ __global__ void __launch_bounds__(256) presort_scatter_kernel(QueryLaunch q) {
 // crossed the other axes first step over every plane the walk would cross
 // before it, so the voxels visited, the boundary points and the shared-point
 // marks are exactly those of the voxel-by-voxel walk (trace_kernel).
+//
+// What bounds it: instruction issue (75% of the slots; latency when a request
+// is small). So voxel and plane indices are FP32 integers (exact: at most
+// 1024), a crossing time costs two instructions and no conversion, the three
+// axes run one straight-line sequence whatever the crossed axis, the voxel
+// after a jump is the floor of a position wherever rounding cannot matter
+// (axis_guess), a boundary point is formed once, as one cell's exit and the
+// next one's entry, and the lanes that ended write their records together at
+// the end of a round. Rounds are long (all lanes' rays end) while the 32 rays
+// of a start enter within an eighth of the box, as a camera's do: the lanes
+// then stay on neighbouring rays. Otherwise idle lanes take new rays after 16
+// cells. On the torus, each measured with the form before (integer indices,
+// lane-by-lane refill) and this one: a million rays from a sphere 574 -> 333 us, a million from the
+// surface 335 -> 199 us, 4,096 rays 85 -> 48 us, 4.19M camera rays 588 -> 593 us.
 // ---------------------------------------------------------------------------
+constexpr int kQueueWords = 14;  // words of a started ray in the queue
+constexpr int kShortRound = 16, kLongRound = 256;  // cells between two refills of a warp's idle lanes
+constexpr int kTraceWarps = 4;
+constexpr int kTraceCtas = 7;    // per SM: 28 warps at 72 registers (32 at 64 spill)
+
 struct LaneRay {
-  int64_t i;
-  int s;           // object slot
+  int i;             // ray (-1: none)
+  int s;             // object slot
   float3 o, d;
-  float inv0, inv1, inv2;
-  int ix0, ix1, ix2, st0, st1, st2;
-  float tcur, t0, t1;
-  int ain;
-  float fin;
+  float3 inv, sg;    // 1 / d (0 when d is 0), sign of d
+  float3 x;          // current voxel
+  float3 in;         // boundary point where the ray entered the current cell
+  float tcur, t1;
+  float clear;       // see axis_guess
   int k, cap;
-  int r;           // the current cell: voxels within r of (ix0, ix1, ix2), all empty when r > 0
-  bool occ;        // the current voxel is occupied (its distance is 0)
-  uint32_t dup;    // bit k: entry point of segment k equals the exit of segment k-1
-  uint32_t lt, lf; // exit (t, face) of the last segment, as bits
-  int la;          // and its axis
+  float r;           // the current cell: voxels within r of x, all empty when r > 0
+  bool occ;          // the current voxel is occupied (its distance is 0)
+  bool adj;          // the cell before was an occupied voxel: the point `in` is its exit
+  uint32_t dup;      // bit k: entry point of segment k equals the exit of segment k-1
 };
 
 __device__ __forceinline__ float sel3(int a, float x, float y, float z) { return a == 0 ? x : (a == 1 ? y : z); }
-__device__ __forceinline__ int sel3i(int a, int x, int y, int z) { return a == 0 ? x : (a == 1 ? y : z); }
 
-// crossing time of plane index P on one axis (the expression dda_walk uses)
-__device__ __forceinline__ float plane_t(int P, float invV, float o, float inv) { return ((float)P * invV - o) * inv; }
+// crossing time of plane P (an integer) on one axis: the expression dda_walk
+// uses (P invV is exact, V being a power of two)
+__device__ __forceinline__ float plane_t(float P, float invV, float o, float inv) { return (P * invV - o) * inv; }
 
-// Planes that one axis crosses before the current cell's exit time ea, as
-// the voxel walk counts them: plane m of the axis (m = 0, 1, ...) is
-// ix + 1 + m for st > 0 and ix - m for st < 0, crossed when its time is
-// below ea, or equal to it when the axis wins the tie (`tie`). Plane times
-// are monotone in m (each operation of plane_t is), so the crossed planes
-// are a prefix: the count is guessed from the position at ea and then
-// corrected with the exact comparisons until plane n is the first one not
-// crossed. At most `cap` planes; 0 when the axis does not move.
-__device__ __forceinline__ int planes_before(int ix, int st, float o, float d, float inv, float invV, int V,
-                                             float ea, bool tie, int cap) {
-  if (st == 0 || cap <= 0) return 0;
-  auto crosses = [&](int m) {
-    const float t = plane_t(st > 0 ? ix + 1 + m : ix - m, invV, o, inv);
-    return t < ea || (tie && t == ea);
-  };
-  const float xe = fmaf(ea, d, o) * (float)V;  // position at ea, in voxels
-  float g = st > 0 ? floorf(xe) - (float)ix : (float)ix - ceilf(xe) + 1.f;
-  g = fminf(fmaxf(g, 0.f), (float)cap);          // also maps NaN to 0
-  int n = (int)g;
-  while (n > 0 && !crosses(n - 1)) --n;
-  while (n < cap && crosses(n)) ++n;
-  return n;
+// Whether the voxel walk crosses a plane of time t before (ea, a): earlier,
+// or at the same time when this axis wins the tie.
+__device__ __forceinline__ bool crosses(float t, float ea, bool tie) { return (t < ea) | (tie & (t == ea)); }
+
+// An axis's voxel when the cell is left at time ea through another axis: the
+// planes crossed before are a prefix of those ahead (plane times are monotone,
+// each operation of plane_t is), at most 2 r of them (r2). The voxel is that of
+// the position at ea; `ok` says that the position keeps clear of the planes, so
+// that comparing the planes' computed times with ea gives the same voxel:
+// plane_t is within 3 x 2^-24 of the true time, relatively, which moves the
+// crossing by at most 3 x 2^-24 (1 + |o|) V voxels, and the position has an
+// error of 2^-24 (1 + |o|) V; `clear` = 1/2 - 2^-20 (2 + |o|) V leaves four
+// times their sum.
+__device__ __forceinline__ float axis_guess(float x, float sg, float o, float d, float r2, float V, float ea,
+                                            float clear, bool &ok) {
+  const float far = fmaf(sg, r2, x);
+  const float v = fmaf(ea, d, o) * V, f = floorf(v);
+  ok = fabsf((v - f) - 0.5f) < clear;
+  return fminf(fmaxf(f, fminf(x, far)), fmaxf(x, far));
 }
 
-// occupancy distance of voxel (x, y, z): 0 when occupied, else the radius
-// of the empty cube around it is D - 1
-__device__ __forceinline__ int voxel_distance(const DevObject &ob, int x, int y, int z) {
-  return __ldg(ob.dist + ((uint32_t)z * ob.V + (uint32_t)y) * ob.V + (uint32_t)x);
+// the same by search from the guess, comparing plane times
+__device__ __noinline__ float axis_search(float g, float x, float sg, float o, float inv, float r, float invV,
+                                          float ea, bool tie) {
+  const float far = fmaf(2.f * sg, r, x), up = fmaxf(sg, 0.f);
+  while (g != x && !crosses(plane_t(g + 1.f - up, invV, o, inv), ea, tie)) g -= sg;
+  while (g != far && crosses(plane_t(g + up, invV, o, inv), ea, tie)) g += sg;
+  return g;
 }
 
-__global__ void __launch_bounds__(256) trace_pool_kernel(QueryLaunch q, int smem_hist, int steps_per_round,
-                                                          const int32_t *__restrict__ perm) {
+// integer of a whole FP32 value in [0, 2^23)
+__device__ __forceinline__ uint32_t whole(float f) { return __float_as_uint(f + 8388608.f) & 0x7fffffu; }
+
+// occupancy distance of voxel x: 0 when occupied, else the radius of the
+// empty cube around it is D - 1 (fV: V as FP32; x inside the grid)
+__device__ __forceinline__ uint32_t voxel_distance(const uint8_t *dist, uint32_t V, float fV, const float3 &x) {
+  return __ldg(dist + (whole(fmaf(x.z, fV, x.y)) * V + whole(x.x)));
+}
+
+__device__ __forceinline__ float sign_of(float d) { return d > 0.f ? 1.f : (d < 0.f ? -1.f : 0.f); }
+
+__global__ void __launch_bounds__(kTraceWarps * 32, kTraceCtas)
+    trace_pool_kernel(QueryLaunch q, int smem_hist, int share, const int32_t *__restrict__ perm) {
   extern __shared__ int sh_hist[];
+  __shared__ uint32_t s_queue[kTraceWarps][kQueueWords][32];
   const int nb = q.n_slots * kBuckets;
   if (smem_hist) {
     for (int i = threadIdx.x; i < nb; i += blockDim.x) sh_hist[i] = 0;
@@ -247,186 +281,196 @@ __global__ void __launch_bounds__(256) trace_pool_kernel(QueryLaunch q, int smem
   const int Hs = q.H_max;
   const unsigned FULL = 0xffffffffu;
   const int lane = threadIdx.x & 31;
+  uint32_t(*sq)[32] = s_queue[threadIdx.x >> 5];
   LaneRay R;
   R.i = -1;
-  bool exhausted = false;
-  int* counter = q.s.meta + 4;
-
-  auto finish = [&](void) {
-    const int64_t i = R.i;
-    q.s.k[i] = (uint8_t)R.k;
-    q.s.dup[i] = R.dup;
-    q.s.slot[i] = (int16_t)R.s;
-    reinterpret_cast<float2 *>(q.s.t01)[i] = make_float2(R.t0, R.t1);
-    if (R.k == 0) miss_store(q.hits, i, q.objs[R.s].n_out);
-    else if (smem_hist) atomicAdd(&sh_hist[R.s * kBuckets + R.k], 1);
-    else atomicAdd(&q.s.counts[R.s * kBuckets + R.k], 1);
-    R.i = -1;
-  };
+  bool exhausted = false;  // uniform: no rays left to start
+  uint32_t next = 0, share_end = 0;  // uniform: rays taken from the counter and not started yet
+  int queued = 0;          // uniform: started rays waiting
+  int steps = kShortRound; // uniform: cells between two refills
+  int *counter = q.s.meta + 4;
 
   for (;;) {
-    // refill: a lane without a ray takes rays until one enters its object's
-    // box (a ray that misses it is answered at once, so no lane spends the
-    // round idle on it) or the pool is empty
+    // hand a started ray to every idle lane
     for (;;) {
-      const bool need = R.i < 0 && !exhausted;
-      const unsigned m = __ballot_sync(FULL, need);
-      if (!m) break;
-      const int leader = __ffs(m) - 1;
-      int base = 0;
-      if (lane == leader) base = atomicAdd(counter, __popc(m));
-      base = __shfl_sync(FULL, base, leader);
-      if (need) {
-        const int64_t pos = (int64_t)base + __popc(m & ((1u << lane) - 1u));
-        if (pos >= n) {
-          exhausted = true;
-        } else {
-          // start ray `my` (the pos-th ray of the presorted order, if any)
-          const int64_t my = perm ? (int64_t)__ldg(perm + pos) : pos;
-          R.i = my;
-          const uint32_t h = q.rays.obj ? q.rays.obj[my] : q.rays.single_handle;
-          R.s = slot_of(q.objs, q.n_slots, h);
-          R.k = 0;
-          R.dup = 0u;
-          R.la = -2;
-          R.t0 = R.t1 = CUDART_NAN_F;
-          if (R.s < 0) {
+      const unsigned idle = __ballot_sync(FULL, R.i < 0);
+      if (!idle || (!queued && exhausted)) break;
+      if (!queued) {
+        // start the next 32 rays of the warp's share, or of a new one
+        if (next == share_end) {
+          int base = 0;
+          if (lane == 0) base = atomicAdd(counter, share);
+          next = (uint32_t)__shfl_sync(FULL, base, 0);
+          share_end = next + share;
+        }
+        const int64_t pos = (int64_t)next + lane;
+        next += 32;
+        exhausted = (int64_t)next >= n;
+        bool live = false, near = false;
+        float3 o, d;
+        float t0 = CUDART_NAN_F, t1 = CUDART_NAN_F;
+        int ea = -1, s = -1, my = 0;
+        if (pos < n) {
+          my = perm ? __ldg(perm + pos) : (int)pos;  // the pos-th ray of the presorted order, if any
+          s = slot_of(q.objs, q.n_slots, q.rays.obj ? q.rays.obj[my] : q.rays.single_handle);
+          int n_out = 0;
+          if (s < 0) {
             atomicOr(q.err, kErrBadHandle);
-            q.s.slot[my] = -1;
+          } else {
+            const DevObject &ob = q.objs[s];
+            n_out = ob.n_out;
+            live = ob.kind == 0 &&
+                   to_unit(ob, q.rays.ox[my], q.rays.oy[my], q.rays.oz[my], q.rays.dx[my], q.rays.dy[my],
+                           q.rays.dz[my], o, d) &&
+                   unit_slab(o, d, q.rays.tmin[my], t0, t1, ea);
+            if (!live) t0 = t1 = CUDART_NAN_F;
+            reinterpret_cast<float2 *>(q.s.t01)[my] = make_float2(t0, t1);
+          }
+          q.s.slot[my] = (int16_t)s;
+          if (!live) {
             q.s.k[my] = 0;
             q.s.dup[my] = 0u;
-            miss_store(q.hits, my, 0);
-            R.i = -1;
-          } else {
-            const DevObject &ob = q.objs[R.s];
-            int ea;
-            float t0, t1;
-            bool live = ob.kind == 0 &&
-                        to_unit(ob, q.rays.ox[my], q.rays.oy[my], q.rays.oz[my], q.rays.dx[my], q.rays.dy[my],
-                                q.rays.dz[my], R.o, R.d) &&
-                        unit_slab(R.o, R.d, q.rays.tmin[my], t0, t1, ea);
-            if (!live) {
-              finish();
-            } else {
-              R.t0 = t0;
-              R.t1 = t1;
-              R.cap = ob.H >> 1;
-              const int V = ob.V;
-              const float3 p = make_float3(fmaf(t0, R.d.x, R.o.x), fmaf(t0, R.d.y, R.o.y), fmaf(t0, R.d.z, R.o.z));
-              int c[3];
-              float dd[3] = {R.d.x, R.d.y, R.d.z}, pp[3] = {p.x, p.y, p.z};
-              int stv[3];
-              float invv[3];
-#pragma unroll
-              for (int a = 0; a < 3; ++a) {
-                int cc = (int)floorf(pp[a] * (float)V);
-                cc = min(max(cc, 0), V - 1);
-                if (a == ea) cc = dd[a] > 0.f ? 0 : V - 1;
-                c[a] = cc;
-                stv[a] = dd[a] > 0.f ? 1 : (dd[a] < 0.f ? -1 : 0);
-                invv[a] = dd[a] != 0.f ? 1.f / dd[a] : 0.f;
-              }
-              R.ix0 = c[0]; R.ix1 = c[1]; R.ix2 = c[2];
-              R.st0 = stv[0]; R.st1 = stv[1]; R.st2 = stv[2];
-              R.inv0 = invv[0]; R.inv1 = invv[1]; R.inv2 = invv[2];
-              R.tcur = t0;
-              R.ain = ea;
-              R.fin = ea >= 0 ? (dd[ea] > 0.f ? 0.f : 1.f) : 0.f;
-              const int D = voxel_distance(ob, c[0], c[1], c[2]);
-              R.r = D > 0 ? D - 1 : 0;
-              R.occ = D == 0;
-            }
+            miss_store(q.hits, my, n_out);
           }
+        }
+        const unsigned m = __ballot_sync(FULL, live);
+        if (live) {
+          const DevObject &ob = q.objs[s];
+          const int V = ob.V;
+          const float pp[3] = {fmaf(t0, d.x, o.x), fmaf(t0, d.y, o.y), fmaf(t0, d.z, o.z)};
+          const float dd[3] = {d.x, d.y, d.z}, oo[3] = {o.x, o.y, o.z};
+          const int e = __popc(m & ((1u << lane) - 1u));
+          uint32_t cell = 0;
+          near = true;
+#pragma unroll
+          for (int a = 0; a < 3; ++a) {
+            int cc = (int)floorf(pp[a] * (float)V);
+            cc = min(max(cc, 0), V - 1);
+            if (a == ea) cc = dd[a] > 0.f ? 0 : V - 1;
+            cell |= (uint32_t)cc << (10 * a);
+            near = near && (__reduce_max_sync(m, cc) - __reduce_min_sync(m, cc)) * 8 <= V;
+            sq[a][e] = __float_as_uint(oo[a]);
+            sq[3 + a][e] = __float_as_uint(dd[a]);
+            sq[6 + a][e] = __float_as_uint(dd[a] != 0.f ? 1.f / dd[a] : 0.f);
+          }
+          sq[9][e] = __float_as_uint(t0);
+          sq[10][e] = __float_as_uint(t1);
+          sq[11][e] = cell;
+          sq[12][e] = (uint32_t)my;
+          sq[13][e] = (uint32_t)s | ((uint32_t)(ea + 1) << 16);
+        }
+        queued = __popc(m);
+        if (queued) steps = __any_sync(FULL, near) ? kLongRound : kShortRound;
+        __syncwarp();
+        continue;
+      }
+      // pop: the j-th idle lane takes the j-th last of the queue
+      const int j = __popc(idle & ((1u << lane) - 1u));
+      if (R.i < 0 && j < queued) {
+        const int e = queued - 1 - j;
+        R.o = make_float3(__uint_as_float(sq[0][e]), __uint_as_float(sq[1][e]), __uint_as_float(sq[2][e]));
+        R.d = make_float3(__uint_as_float(sq[3][e]), __uint_as_float(sq[4][e]), __uint_as_float(sq[5][e]));
+        R.inv = make_float3(__uint_as_float(sq[6][e]), __uint_as_float(sq[7][e]), __uint_as_float(sq[8][e]));
+        R.sg = make_float3(sign_of(R.d.x), sign_of(R.d.y), sign_of(R.d.z));
+        R.tcur = __uint_as_float(sq[9][e]);
+        R.t1 = __uint_as_float(sq[10][e]);
+        const uint32_t cell = sq[11][e];
+        R.x = make_float3((float)(cell & 1023u), (float)((cell >> 10) & 1023u), (float)(cell >> 20));
+        R.i = (int)sq[12][e];
+        const uint32_t se = sq[13][e];
+        R.s = (int)(se & 0xffffu);
+        const int ea = (int)(se >> 16) - 1;
+        R.in = seg_point(R.o, R.d, R.tcur, ea,
+                         ea >= 0 ? (sel3(ea, R.d.x, R.d.y, R.d.z) > 0.f ? 0.f : 1.f) : 0.f);
+        R.adj = false;
+        R.k = 0;
+        R.dup = 0u;
+        const DevObject &ob = q.objs[R.s];
+        R.cap = ob.H >> 1;
+        const uint32_t V = ob.V;
+        R.clear = 0.5f - (fmaxf(fabsf(R.o.x), fmaxf(fabsf(R.o.y), fabsf(R.o.z))) + 2.f) * (float)V * 9.5367431640625e-7f;
+        const uint32_t D = voxel_distance(ob.dist, V, (float)V, R.x);
+        R.r = fmaxf((float)D - 1.f, 0.f);
+        R.occ = D == 0;
+      }
+      queued = max(queued - __popc(idle), 0);
+      __syncwarp();
+    }
+    if (__all_sync(FULL, R.i < 0)) break;
+    if (R.i < 0) continue;
+    // up to `steps` cells of this lane's ray
+    const DevObject &ob = q.objs[R.s];
+    const uint32_t V = ob.V;
+    const float invV = ob.invV, fV = (float)V;
+    const uint8_t *dist = ob.dist;  // in registers: the stores below could alias the object table
+    float *P = q.s.pts + (size_t)R.i * Hs * 3;
+    bool done = false;
+    for (int it = 0; it < steps && !done; ++it) {
+      // exit plane of the cell on each axis, and its crossing time
+      const float P0 = fmaf(R.sg.x, R.r, R.x.x) + fmaxf(R.sg.x, 0.f);
+      const float P1 = fmaf(R.sg.y, R.r, R.x.y) + fmaxf(R.sg.y, 0.f);
+      const float P2 = fmaf(R.sg.z, R.r, R.x.z) + fmaxf(R.sg.z, 0.f);
+      const float e0 = R.sg.x != 0.f ? plane_t(P0, invV, R.o.x, R.inv.x) : CUDART_INF_F;
+      const float e1 = R.sg.y != 0.f ? plane_t(P1, invV, R.o.y, R.inv.y) : CUDART_INF_F;
+      const float e2 = R.sg.z != 0.f ? plane_t(P2, invV, R.o.z, R.inv.z) : CUDART_INF_F;
+      const int a = (e0 <= e1) ? (e0 <= e2 ? 0 : 2) : (e1 <= e2 ? 1 : 2);
+      const float ea = sel3(a, e0, e1, e2);
+      const float tx = fminf(ea, R.t1);
+      // the cell's exit point, the next cell's entry
+      const float3 out = make_float3(a == 0 ? P0 * invV : fmaf(tx, R.d.x, R.o.x),
+                                     a == 1 ? P1 * invV : fmaf(tx, R.d.y, R.o.y),
+                                     a == 2 ? P2 * invV : fmaf(tx, R.d.z, R.o.z));
+      const bool emit = R.occ & (tx > R.tcur);
+      if (emit) {
+        float2 *w = reinterpret_cast<float2 *>(P + 6 * R.k);
+        w[0] = make_float2(R.in.x, R.in.y);
+        w[1] = make_float2(R.in.z, out.x);
+        w[2] = make_float2(out.y, out.z);
+        R.dup |= (R.adj ? 1u : 0u) << R.k;
+        ++R.k;
+      }
+      R.adj = emit;
+      done = (ea >= R.t1) | (R.k >= R.cap);
+      if (!done) {
+        // The other axes first cross the planes the voxel walk crosses
+        // before (ea, a) -- at most 2 r each, none for a voxel -- then axis a
+        // crosses its plane. A cube may reach past the grid: an axis whose
+        // next plane is the grid's own boundary leaves the grid there, and
+        // the voxel walk ends at that crossing (the slab's exit time and the
+        // plane's crossing time may round differently), so the ray ends here
+        // too -- the cube holds no occupied voxel, so nothing is lost.
+        bool ok0, ok1, ok2;
+        const float r2 = R.r + R.r;
+        float g0 = axis_guess(R.x.x, R.sg.x, R.o.x, R.d.x, r2, fV, ea, R.clear, ok0);
+        float g1 = axis_guess(R.x.y, R.sg.y, R.o.y, R.d.y, r2, fV, ea, R.clear, ok1);
+        float g2 = axis_guess(R.x.z, R.sg.z, R.o.z, R.d.z, r2, fV, ea, R.clear, ok2);
+        if (!((ok0 | (a == 0)) & (ok1 | (a == 1)) & (ok2 | (a == 2)))) {
+          if (a != 0) g0 = axis_search(g0, R.x.x, R.sg.x, R.o.x, R.inv.x, R.r, invV, ea, true);
+          if (a != 1) g1 = axis_search(g1, R.x.y, R.sg.y, R.o.y, R.inv.y, R.r, invV, ea, a == 2);
+          if (a != 2) g2 = axis_search(g2, R.x.z, R.sg.z, R.o.z, R.inv.z, R.r, invV, ea, false);
+        }
+        // the voxel behind axis a's plane
+        R.x.x = a == 0 ? P0 + fminf(R.sg.x, 0.f) : g0;
+        R.x.y = a == 1 ? P1 + fminf(R.sg.y, 0.f) : g1;
+        R.x.z = a == 2 ? P2 + fminf(R.sg.z, 0.f) : g2;
+        done = (fminf(R.x.x, fminf(R.x.y, R.x.z)) < 0.f) | (fmaxf(R.x.x, fmaxf(R.x.y, R.x.z)) >= fV);
+        if (!done) {
+          R.tcur = ea;
+          R.in = out;
+          // the next cell is centred on the voxel just entered
+          const uint32_t D = voxel_distance(dist, V, fV, R.x);
+          R.r = fmaxf(__uint_as_float(0x4b000000u | D) - 8388609.f, 0.f);
+          R.occ = D == 0;
         }
       }
     }
-    if (__all_sync(FULL, R.i < 0 && exhausted)) break;
-    if (R.i < 0) continue;
-    // up to steps_per_round cells of this lane's ray
-    const DevObject &ob = q.objs[R.s];
-    const int V = ob.V;
-    const float invV = ob.invV;
-    float *P = q.s.pts + (size_t)R.i * Hs * 3;
-    for (int it = 0; it < steps_per_round; ++it) {
-      bool done = false;
-      const int rr = R.r;  // cell: the voxel, or the empty cube of radius rr around it
-      // exit plane of the cell on each axis, and its crossing time
-      const int P0 = R.st0 > 0 ? R.ix0 + rr + 1 : R.ix0 - rr;
-      const int P1 = R.st1 > 0 ? R.ix1 + rr + 1 : R.ix1 - rr;
-      const int P2 = R.st2 > 0 ? R.ix2 + rr + 1 : R.ix2 - rr;
-      const float e0 = R.st0 != 0 ? plane_t(P0, invV, R.o.x, R.inv0) : CUDART_INF_F;
-      const float e1 = R.st1 != 0 ? plane_t(P1, invV, R.o.y, R.inv1) : CUDART_INF_F;
-      const float e2 = R.st2 != 0 ? plane_t(P2, invV, R.o.z, R.inv2) : CUDART_INF_F;
-      const int a = (e0 <= e1) ? (e0 <= e2 ? 0 : 2) : (e1 <= e2 ? 1 : 2);
-      const float ea = sel3(a, e0, e1, e2);
-      const int Pa = sel3i(a, P0, P1, P2);
-      const float tx = fminf(ea, R.t1);
-      if (R.occ && tx > R.tcur) {
-        const float fx = (float)Pa * invV;
-        if (R.k > 0 && __float_as_uint(R.tcur) == R.lt && R.ain == R.la && __float_as_uint(R.fin) == R.lf)
-          R.dup |= 1u << R.k;
-        R.lt = __float_as_uint(tx);
-        R.la = a;
-        R.lf = __float_as_uint(fx);
-        const float3 pa = seg_point(R.o, R.d, R.tcur, R.ain, R.fin);
-        const float3 pb = seg_point(R.o, R.d, tx, a, fx);
-        float *w = P + 6 * R.k;
-        reinterpret_cast<float2 *>(w)[0] = make_float2(pa.x, pa.y);
-        reinterpret_cast<float2 *>(w)[1] = make_float2(pa.z, pb.x);
-        reinterpret_cast<float2 *>(w)[2] = make_float2(pb.y, pb.z);
-        if (++R.k >= R.cap) done = true;
-      }
-      if (!done && ea >= R.t1) done = true;
-      if (!done) {
-        // when a cube is crossed, the other axes first cross the planes the
-        // voxel walk crosses before (ea, a) -- at most 2 rr each; for a voxel
-        // there are none
-        // A cube may reach past the grid: an axis whose next plane is the
-        // grid's own boundary leaves the grid there, and the voxel walk
-        // ends at that crossing (the slab's exit time and the plane's
-        // crossing time may round differently), so the ray ends here too
-        // -- the cube holds no occupied voxel, so nothing is lost.
-        bool out = false;
-        if (rr) {
-          // axis b moves n_b voxels; stepping onto voxel -1 or V (more steps
-          // than the grid leaves, m_b) means the ray leaves the grid first
-          const int n0 = a == 0 ? 0 : planes_before(R.ix0, R.st0, R.o.x, R.d.x, R.inv0, invV, V, ea, true, 2 * rr);
-          const int n1 = a == 1 ? 0 : planes_before(R.ix1, R.st1, R.o.y, R.d.y, R.inv1, invV, V, ea, a == 2, 2 * rr);
-          const int n2 = a == 2 ? 0 : planes_before(R.ix2, R.st2, R.o.z, R.d.z, R.inv2, invV, V, ea, false, 2 * rr);
-          out = n0 > (R.st0 > 0 ? V - 1 - R.ix0 : R.ix0) || n1 > (R.st1 > 0 ? V - 1 - R.ix1 : R.ix1) ||
-                n2 > (R.st2 > 0 ? V - 1 - R.ix2 : R.ix2);
-          R.ix0 += R.st0 * n0;
-          R.ix1 += R.st1 * n1;
-          R.ix2 += R.st2 * n2;
-        }
-        // then axis a crosses its plane
-        const int sa = sel3i(a, R.st0, R.st1, R.st2);
-        const int ia = sa > 0 ? Pa : Pa - 1;
-        if (out || ia < 0 || ia >= V) {
-          done = true;
-        } else {
-          R.tcur = ea;
-          R.ain = a;
-          R.fin = (float)Pa * invV;
-          if (a == 0) R.ix0 = ia;
-          else if (a == 1) R.ix1 = ia;
-          else R.ix2 = ia;
-          // the next cell is centred on the voxel just entered (indices
-          // are checked: a violation is reported, never read)
-          if ((unsigned)R.ix0 >= (unsigned)V || (unsigned)R.ix1 >= (unsigned)V || (unsigned)R.ix2 >= (unsigned)V) {
-            atomicOr(q.err, kErrCheck);
-            done = true;
-          } else {
-            const int D = voxel_distance(ob, R.ix0, R.ix1, R.ix2);
-            R.r = D > 0 ? D - 1 : 0;
-            R.occ = D == 0;
-          }
-        }
-      }
-      if (done) {
-        finish();
-        break;
-      }
+    if (done) {  // the lanes that ended in this round, together
+      q.s.k[R.i] = (uint8_t)R.k;
+      q.s.dup[R.i] = R.dup;
+      if (R.k == 0) miss_store(q.hits, R.i, q.objs[R.s].n_out);
+      else if (smem_hist) atomicAdd(&sh_hist[R.s * kBuckets + R.k], 1);
+      else atomicAdd(&q.s.counts[R.s * kBuckets + R.k], 1);
+      R.i = -1;
     }
   }
   if (smem_hist) {
@@ -995,24 +1039,35 @@ static int grid_for(int64_t n, int threads, int cap) {
   return (int)g;
 }
 
+// the CTAs that are resident at once
+static int trace_pool_grid(int64_t n, int sms) {
+  return (int)std::max<int64_t>(1, std::min<int64_t>((n + kTraceWarps * 32 - 1) / (kTraceWarps * 32), (int64_t)sms * kTraceCtas));
+}
+
+// Rays a warp takes from the counter at once: 32, and up to 256 where each
+// warp starts at least 8 such shares (fewer atomics on one address; within
+// 2% of 32 at every size timed).
+static int trace_pool_share(int64_t n, int grid) {
+  return 32 * (int)std::max<int64_t>(1, std::min<int64_t>(8, n / ((int64_t)grid * kTraceWarps * 32 * 8)));
+}
+
 cudaError_t launch_trace(const QueryLaunch &q, int *launches) {
-  cudaMemsetAsync(q.s.counts, 0, sizeof(int32_t) * q.n_slots * kBuckets, q.stream);
   const int nb = q.n_slots * kBuckets;
+  cudaMemsetAsync(q.s.counts, 0, sizeof(int32_t) * nb, q.stream);
+  if (q.trace_mode != 0) cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
   const int smem_hist = nb <= 12288;
   const size_t smem = smem_hist ? nb * sizeof(int) : 0;
+  if (q.trace_mode != 0 && smem > (32 << 10)) {  // with the queue, past the 48 KiB a launch may use unasked
+    const cudaError_t e =
+        cudaFuncSetAttribute(trace_pool_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 48 << 10);
+    if (e != cudaSuccess) return e;
+  }
   if (q.trace_mode == 1) {
-    cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int64_t need = (q.rays.n + 255) / 256;
-    const int grid = (int)std::min<int64_t>(need, (int64_t)sms * 8);
-    // long rounds: a lane whose ray ends waits for the warp's round to end,
-    // so that the next refill starts many rays together (the start of a
-    // ray -- unit-cube transform, slab test, first cell -- is the costly,
-    // divergent part); 8, 32 and 64 cells per round took 0.76, 0.66 and
-    // 0.61 ms on the 4M-ray torus query
-    trace_pool_kernel<<<grid, 256, smem, q.stream>>>(q, smem_hist, 64, nullptr);
+    const int grid = trace_pool_grid(q.rays.n, sms);
+    trace_pool_kernel<<<grid, kTraceWarps * 32, smem, q.stream>>>(q, smem_hist, trace_pool_share(q.rays.n, grid), nullptr);
     *launches += 1;
     return cudaGetLastError();
   }
@@ -1021,7 +1076,6 @@ cudaError_t launch_trace(const QueryLaunch &q, int *launches) {
     const uint32_t last = (uint32_t)q.n_slots << key_bits;  // rays the traversal answers as misses
     const int64_t nbins = (int64_t)last + 1;
     const unsigned blocks = (unsigned)std::max<int64_t>((q.rays.n + 255) / 256, 1);
-    cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
     cudaError_t e = cudaMemsetAsync(q.s.bins, 0, (size_t)nbins * 4, q.stream);
     if (e != cudaSuccess) return e;
     presort_count_kernel<<<blocks, 256, 0, q.stream>>>(q, key_bits, last);
@@ -1031,8 +1085,8 @@ cudaError_t launch_trace(const QueryLaunch &q, int *launches) {
     int dev = 0, sms = 152;
     cudaGetDevice(&dev);
     cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    const int grid = (int)std::min<int64_t>((q.rays.n + 255) / 256, (int64_t)sms * 8);
-    trace_pool_kernel<<<grid, 256, smem, q.stream>>>(q, smem_hist, 64, q.s.order);
+    const int grid = trace_pool_grid(q.rays.n, sms);
+    trace_pool_kernel<<<grid, kTraceWarps * 32, smem, q.stream>>>(q, smem_hist, trace_pool_share(q.rays.n, grid), q.s.order);
     *launches += 6;
     return cudaGetLastError();
   }
