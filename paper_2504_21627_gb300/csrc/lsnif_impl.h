@@ -15,6 +15,8 @@ constexpr uint32_t kPi2 = 2654435761u;
 constexpr uint32_t kPi3 = 805459861u;
 
 constexpr int kMaxCap = 32;          // H/2 <= 32
+constexpr int kMaxObjects = 1024;    // object slots of a context
+constexpr int kMetaWords = 64;       // words of QueryScratch::meta
 constexpr int kBuckets = kMaxCap + 1;  // per object: k = 0..32
 constexpr int kTileM = 128;          // rays per tensor-core tile (tcgen05 M)
 constexpr int kDistCap = 32;         // largest stored occupancy distance

@@ -132,11 +132,11 @@ extern "C" int lsnif_query_rays_noalloc(lsnif_ctx *ctx, const lsnif_rays *r, lsn
   s.dup = reinterpret_cast<uint32_t *>(take((size_t)n * 4));
   s.slot = reinterpret_cast<int16_t *>(take((size_t)n * 2));
   s.order = reinterpret_cast<int32_t *>(take((size_t)n * 4));
+  s.meta = reinterpret_cast<int32_t *>(take(kMetaWords * 4));
   s.counts = reinterpret_cast<int32_t *>(take((size_t)n_slots * kBuckets * 4));
   s.offsets = reinterpret_cast<int32_t *>(take((size_t)n_slots * kBuckets * 4));
   s.cursor = reinterpret_cast<int32_t *>(take((size_t)n_slots * kBuckets * 4));
   s.tiles = reinterpret_cast<int32_t *>(take((size_t)max_tiles * 12));
-  s.meta = reinterpret_cast<int32_t *>(take(64 * 4));
   s.blk = reinterpret_cast<int32_t *>(take((size_t)(n / kGroupBlock + 2) * 8));
   if (spatial) {
     s.bins = reinterpret_cast<int32_t *>(take((size_t)kBinsAlloc * 4));

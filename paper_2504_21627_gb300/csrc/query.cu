@@ -480,43 +480,81 @@ __global__ void __launch_bounds__(kTraceWarps * 32, kTraceCtas)
   }
 }
 
+// Exclusive scan of one value per thread over a block of 1024; `total` is the
+// block's sum. ws: 33 words of shared memory, free again when the call returns.
+__device__ __forceinline__ int block_scan(int v, int *ws, int &total) {
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  int inc = v;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int y = __shfl_up_sync(0xffffffffu, inc, o);
+    if (lane >= o) inc += y;
+  }
+  if (lane == 31) ws[w] = inc;
+  __syncthreads();
+  if (w == 0) {
+    int x = ws[lane];
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+      const int y = __shfl_up_sync(0xffffffffu, x, o);
+      if (lane >= o) x += y;
+    }
+    ws[lane] = x;
+  }
+  __syncthreads();
+  const int before = (w ? ws[w - 1] : 0) + inc - v;
+  total = ws[31];
+  __syncthreads();
+  return before;
+}
+
 // Single block: bucket offsets (object ascending, k descending), tiles of
-// kTileM rays that never straddle objects, totals, cursors reset.
+// kTileM rays that never straddle objects, totals, cursors reset. A warp takes
+// one object's 32 buckets at a time, so an object's range starts at the value
+// its lane 0 scans to. One thread walking the buckets took 11 us on one object
+// (a load per bucket, none in flight beside another) and grew with the
+// objects; this takes 3 us, the launch included.
 __global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
-  __shared__ int tile_off[1025];
-  __shared__ int obj_live[1024];
+  __shared__ int ws[33];
+  __shared__ int first[kMaxObjects + 1];     // start of each object's range
+  __shared__ int tile_off[kMaxObjects + 1];  // and its first tile
   const int ns = q.n_slots;
+  static_assert(kMaxCap == 32, "a warp per object");
+  int run = 0, pts = 0;
+  for (int base = 0; base < ns * kMaxCap; base += 1024) {
+    const int s = (base + (int)threadIdx.x) >> 5, k = kMaxCap - (threadIdx.x & 31);
+    const int c = s < ns ? q.s.counts[s * kBuckets + k] : 0;
+    int total;
+    const int at = run + block_scan(c, ws, total);
+    // group modes 2 and 3: one bucket per object (bucket k = 1 takes all)
+    const int start = __shfl_sync(0xffffffffu, at, 0);
+    if (s < ns) {
+      q.s.offsets[s * kBuckets + k] = q.group_mode >= 2 ? start : at;
+      q.s.cursor[s * kBuckets + k] = 0;
+      if (k == kMaxCap) first[s] = at;
+    }
+    pts += 2 * k * c;
+    run += total;
+  }
+  int points;
+  block_scan(pts, ws, points);  // also a barrier: first[] is written
+  if (threadIdx.x == 0) first[ns] = run;
+  __syncthreads();
+  const int live = (int)threadIdx.x < ns ? first[threadIdx.x + 1] - first[threadIdx.x] : 0;
+  int tiles;
+  const int tile0 = block_scan((live + kTileM - 1) / kTileM, ws, tiles);
+  if ((int)threadIdx.x < ns) tile_off[threadIdx.x] = tile0;
+  if (tiles > q.s.max_tiles) {
+    if (threadIdx.x == 0) atomicOr(q.err, kErrCheck);
+    tiles = q.s.max_tiles;
+  }
   if (threadIdx.x == 0) {
-    int run = 0, tiles = 0, pts = 0;
-    for (int s = 0; s < ns; ++s) {
-      int start = run;
-      for (int k = kMaxCap; k >= 1; --k) {
-        int c = q.s.counts[s * kBuckets + k];
-        // group modes 2 and 3: one bucket per object (bucket k = 1 takes all)
-        q.s.offsets[s * kBuckets + k] = q.group_mode >= 2 ? start : run;
-        q.s.cursor[s * kBuckets + k] = 0;
-        run += c;
-        pts += 2 * k * c;
-      }
-      int live = run - start;
-      if (s < 1024) {
-        obj_live[s] = start;  // start of the object's range
-        tile_off[s] = tiles;
-      }
-      tiles += (live + kTileM - 1) / kTileM;
-    }
-    if (ns <= 1024) tile_off[ns] = tiles;
-    if (tiles > q.s.max_tiles) {
-      atomicOr(q.err, kErrCheck);
-      tiles = q.s.max_tiles;
-    }
     q.s.meta[0] = run;
     q.s.meta[1] = tiles;
-    q.s.meta[2] = pts;
+    q.s.meta[2] = points;
     q.s.meta[3] = 0;
   }
   __syncthreads();
-  const int tiles = q.s.meta[1];
   for (int t = threadIdx.x; t < tiles; t += blockDim.x) {
     // object of tile t: last s with tile_off[s] <= t
     int lo = 0, hi = ns - 1;
@@ -524,15 +562,10 @@ __global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
       int mid = (lo + hi + 1) >> 1;
       if (tile_off[mid] <= t) lo = mid; else hi = mid - 1;
     }
-    int s = lo;
-    int first = obj_live[s];
-    int obj_end = first;
-    for (int k = 1; k <= kMaxCap; ++k) obj_end += q.s.counts[s * kBuckets + k];
-    int start = first + (t - tile_off[s]) * kTileM;
-    int cnt = min(kTileM, obj_end - start);
-    q.s.tiles[3 * t + 0] = s;
+    const int start = first[lo] + (t - tile_off[lo]) * kTileM;
+    q.s.tiles[3 * t + 0] = lo;
     q.s.tiles[3 * t + 1] = start;
-    q.s.tiles[3 * t + 2] = cnt;
+    q.s.tiles[3 * t + 2] = min(kTileM, first[lo + 1] - start);
   }
 }
 
@@ -638,41 +671,30 @@ __global__ void __launch_bounds__(1024) group_count_kernel(QueryLaunch q, int nb
 }
 
 __global__ void __launch_bounds__(1024) group_scan_kernel(QueryLaunch q, int nblk) {
-  __shared__ int s_part[1024];
-  __shared__ int s_pts[1024];
+  __shared__ int ws[33];
   const int per = (nblk + 1023) / 1024;
   const int b0 = threadIdx.x * per;
   int sum = 0, pts = 0;
   for (int b = b0; b < min(b0 + per, nblk); ++b) { sum += q.s.blk[b]; pts += q.s.blk[nblk + b]; }
-  s_part[threadIdx.x] = sum;
-  s_pts[threadIdx.x] = pts;
-  __syncthreads();
-  if (threadIdx.x == 0) {   // exclusive scan of the 1024 partial sums
-    int run = 0, pr = 0;
-    for (int t = 0; t < 1024; ++t) {
-      const int v = s_part[t];
-      s_part[t] = run;
-      run += v;
-      pr += s_pts[t];
-    }
-    int tiles = (run + kTileM - 1) / kTileM;
-    if (tiles > q.s.max_tiles) {
-      atomicOr(q.err, kErrCheck);
-      tiles = q.s.max_tiles;
-    }
-    q.s.meta[0] = run;
+  int n_live, points;
+  int run = block_scan(sum, ws, n_live);
+  block_scan(pts, ws, points);
+  int tiles = (n_live + kTileM - 1) / kTileM;
+  if (tiles > q.s.max_tiles) {
+    if (threadIdx.x == 0) atomicOr(q.err, kErrCheck);
+    tiles = q.s.max_tiles;
+  }
+  if (threadIdx.x == 0) {
+    q.s.meta[0] = n_live;
     q.s.meta[1] = tiles;
-    q.s.meta[2] = pr;
+    q.s.meta[2] = points;
     q.s.meta[3] = 0;
   }
-  __syncthreads();
-  int run = s_part[threadIdx.x];
   for (int b = b0; b < min(b0 + per, nblk); ++b) {   // block offsets replace the counts
     const int v = q.s.blk[b];
     q.s.blk[b] = run;
     run += v;
   }
-  const int n_live = q.s.meta[0], tiles = q.s.meta[1];
   for (int t = threadIdx.x; t < tiles; t += blockDim.x) {
     q.s.tiles[3 * t + 0] = q.single_slot;
     q.s.tiles[3 * t + 1] = t * kTileM;
@@ -680,30 +702,42 @@ __global__ void __launch_bounds__(1024) group_scan_kernel(QueryLaunch q, int nbl
   }
 }
 
+// A block's 4 x 1024 rays: every thread reads its four first, then one scan
+// over the (round, warp) totals places them in ray order.
 __global__ void __launch_bounds__(1024) group_scatter_kernel(QueryLaunch q) {
-  __shared__ int s_warp[32];
-  __shared__ int s_total;
+  constexpr int kRounds = kGroupBlock / 1024;
+  __shared__ int s_off[kRounds * 32];
   const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  int base = q.s.blk[b];
-  for (int r = 0; r < kGroupBlock / 1024; ++r) {
+  const int base = q.s.blk[b];
+  unsigned m[kRounds];
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
     const int64_t i = (int64_t)b * kGroupBlock + r * 1024 + threadIdx.x;
-    const bool live = i < q.rays.n && q.s.slot[i] >= 0 && q.s.k[i] > 0;
-    const unsigned m = __ballot_sync(0xffffffffu, live);
-    if (lane == 0) s_warp[warp] = __popc(m);
-    __syncthreads();
-    if (threadIdx.x == 0) {
-      int run = 0;
-      for (int w = 0; w < 32; ++w) {
-        const int v = s_warp[w];
-        s_warp[w] = run;
-        run += v;
+    m[r] = __ballot_sync(0xffffffffu, i < q.rays.n && q.s.slot[i] >= 0 && q.s.k[i] > 0);
+    if (lane == 0) s_off[r * 32 + warp] = __popc(m[r]);
+  }
+  __syncthreads();
+  if (warp == 0) {  // exclusive scan of the kRounds x 32 totals
+    int run = 0;
+#pragma unroll
+    for (int r = 0; r < kRounds; ++r) {
+      const int v = s_off[r * 32 + lane];
+      int inc = v;
+#pragma unroll
+      for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, inc, o);
+        if (lane >= o) inc += y;
       }
-      s_total = run;
+      s_off[r * 32 + lane] = run + inc - v;
+      run += __shfl_sync(0xffffffffu, inc, 31);
     }
-    __syncthreads();
-    if (live) q.s.order[base + s_warp[warp] + __popc(m & ((1u << lane) - 1u))] = (int32_t)i;
-    base += s_total;
-    __syncthreads();
+  }
+  __syncthreads();
+#pragma unroll
+  for (int r = 0; r < kRounds; ++r) {
+    const int64_t i = (int64_t)b * kGroupBlock + r * 1024 + threadIdx.x;
+    if ((m[r] >> lane) & 1u)
+      q.s.order[base + s_off[r * 32 + warp] + __popc(m[r] & ((1u << lane) - 1u))] = (int32_t)i;
   }
 }
 
@@ -1053,8 +1087,12 @@ static int trace_pool_share(int64_t n, int grid) {
 
 cudaError_t launch_trace(const QueryLaunch &q, int *launches) {
   const int nb = q.n_slots * kBuckets;
-  cudaMemsetAsync(q.s.counts, 0, sizeof(int32_t) * nb, q.stream);
-  if (q.trace_mode != 0) cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
+  // the counters and the histogram, in one operation where they lie together
+  const bool joined = q.s.counts == q.s.meta + kMetaWords;
+  cudaError_t e0 = cudaMemsetAsync(joined ? q.s.meta : q.s.counts, 0,
+                                   sizeof(int32_t) * (nb + (joined ? kMetaWords : 0)), q.stream);
+  if (e0 == cudaSuccess && !joined) e0 = cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
+  if (e0 != cudaSuccess) return e0;
   const int smem_hist = nb <= 12288;
   const size_t smem = smem_hist ? nb * sizeof(int) : 0;
   if (q.trace_mode != 0 && smem > (32 << 10)) {  // with the queue, past the 48 KiB a launch may use unasked

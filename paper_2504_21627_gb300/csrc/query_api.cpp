@@ -87,12 +87,12 @@ static QueryScratch carve(Workspace *ws, int64_t n, int H, int n_slots, int n_in
   s.dup = c.take<uint32_t>((size_t)N * 4);
   s.slot = c.take<int16_t>((size_t)N * 2);
   s.order = c.take<int32_t>((size_t)N * 4);
+  s.meta = c.take<int32_t>(kMetaWords * 4);  // 256 bytes: counts follow at once (cleared together)
   s.counts = c.take<int32_t>((size_t)SS * kBuckets * 4);
   s.offsets = c.take<int32_t>((size_t)SS * kBuckets * 4);
   s.cursor = c.take<int32_t>((size_t)SS * kBuckets * 4);
   const int mt = max_tiles_for(N, SS);
   s.tiles = c.take<int32_t>((size_t)mt * 12);
-  s.meta = c.take<int32_t>(64 * 4);
   s.blk = c.take<int32_t>((size_t)(N / kGroupBlock + 2) * 8);
   s.bins = c.take<int32_t>((size_t)kBinsAlloc * 4);
   s.bin_sums = c.take<int32_t>((size_t)kBinSumsAlloc * 4);

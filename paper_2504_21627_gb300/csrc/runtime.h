@@ -14,7 +14,7 @@
 
 namespace lsnif {
 
-constexpr int kMaxSlots = 1024;
+constexpr int kMaxSlots = kMaxObjects;
 
 struct Object {
   lsnif_config cfg{};
