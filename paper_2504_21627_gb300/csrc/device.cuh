@@ -154,6 +154,8 @@ __device__ __forceinline__ uint32_t pick4(const uint4 &g, uint32_t j) {
 }
 
 // Decode of the network outputs (Sec. 5.1, 5.3) for one ray and its stores.
+// NZ: largest n_out; 16 unrolls the loops over z, which then stays in registers.
+template <int NZ = 64>
 __device__ __forceinline__ void decode_store(const HitsArg &h, int64_t ray, const float *z, int n_out, int n_mat,
                                              float t0, float t1, float tmin, float tmax) {
   bool occ = z[0] > 0.f;
@@ -163,8 +165,14 @@ __device__ __forceinline__ void decode_store(const HitsArg &h, int64_t ray, cons
   if (nn > 0.f) { float r = 1.f / nn; nx *= r; ny *= r; nz *= r; } else { nx = ny = nz = 0.f; }
   int best = 0;
   float bv = z[8];
-  for (int m = 1; m < n_mat; ++m)
-    if (z[8 + m] > bv) { bv = z[8 + m]; best = m; }
+  if constexpr (NZ == 16) {
+#pragma unroll
+    for (int m = 1; m < 8; ++m)
+      if (m < n_mat && z[8 + m] > bv) { bv = z[8 + m]; best = m; }
+  } else {
+    for (int m = 1; m < n_mat; ++m)
+      if (z[8 + m] > bv) { bv = z[8 + m]; best = m; }
+  }
   bool hit = occ && t >= tmin && t <= tmax;
   if (h.hit) h.hit[ray] = hit ? 1 : 0;
   if (h.t) h.t[ray] = t;
@@ -175,8 +183,15 @@ __device__ __forceinline__ void decode_store(const HitsArg &h, int64_t ray, cons
   if (h.ar) h.ar[ray] = sigmoidf_(z[5]);
   if (h.ag) h.ag[ray] = sigmoidf_(z[6]);
   if (h.ab) h.ab[ray] = sigmoidf_(z[7]);
-  if (h.logits)
-    for (int j = 0; j < n_out; ++j) h.logits[ray * n_out + j] = z[j];
+  if (h.logits) {
+    if constexpr (NZ == 16) {
+#pragma unroll
+      for (int j = 0; j < 16; ++j)
+        if (j < n_out) h.logits[ray * n_out + j] = z[j];
+    } else {
+      for (int j = 0; j < n_out; ++j) h.logits[ray * n_out + j] = z[j];
+    }
+  }
 }
 
 __device__ __forceinline__ void miss_store(const HitsArg &h, int64_t ray, int n_out) {

@@ -7,30 +7,37 @@
 // FP16 (kind::f16 takes either, A and B always of the same type); FP32
 // accumulation in both.
 //
-// Work unit: a tile of 128 rays (the tcgen05 M). The first layer's K runs
-// over the tile's occupied-voxel segments: chunk s holds the features of
-// points 2s and 2s+1 (2*L*F 16-bit columns, no-swizzle K-major core-matrix
-// layout). Chunks no ray of the tile reaches are skipped (tiles are sorted
-// by point count).
+// Work unit: a tile of up to 128 rays (the tcgen05 M; 64 or 32 rows of one
+// when the rays are few). The first layer's K runs over the tile's
+// occupied-voxel segments: chunk s holds the features of points 2s and 2s+1
+// (2*L*F 16-bit columns, no-swizzle K-major core-matrix layout). Chunks no ray
+// of the tile reaches are skipped.
 //
 // Warp roles:
-//   gather warps (NG): build the tile's work lists, then fill chunk after
-//     chunk into a ring of shared-memory A tiles;
+//   gather warps (NG): fill chunk after chunk into a ring of shared-memory A
+//     tiles;
 //   one MMA warp: issues each filled chunk's MMAs against the resident
 //     first-layer weights into the tile's TMEM accumulator;
-//   four epilogue warps (TMEM lane = ray): hidden and output layers (bias,
-//     activation, 16-bit activations back to shared memory, next MMA) and the
-//     decode, while the gather warps fill the next tile. Two TMEM
-//     accumulators alternate between tiles.
+//   four epilogue warps (TMEM lane = ray): set the next tile up (rows, work
+//     lists), then hidden and output layers (bias, activation, 16-bit
+//     activations back to tensor memory, next MMA) and the decode, while the
+//     gather warps fill the next tile. Two TMEM accumulators alternate
+//     between tiles.
 //
-// Shared boundary points: consecutive occupied voxels along a ray share a
-// face, and the traversal marks an entry point that is bit-identical to the
-// previous segment's exit (bit s of the ray's dup mask). Such a point is
-// gathered once: its chunk copies the features from the previous chunk's A
-// tile. A chunk's work is thus a list of gathers, copies and zero fills (two
-// entries per ray); gathers go round-robin over the gather warps in blocks
-// of 32 items (item = one point x one 16-byte column group), so every warp
-// gets the same share whatever the mix.
+// Rows without a segment s take no part in chunk s: the MMAs leave their
+// accumulators as they are (disable-output-lane masks), so nothing is written
+// for them. Shared boundary points: consecutive occupied voxels along a ray
+// share a face, and the traversal marks an entry point that is bit-identical
+// to the previous segment's exit (bit s of the ray's dup mask). Such a point
+// is gathered once: the MMAs of its chunk's entry half read the previous
+// chunk's exit half for the marked rows, and this chunk's entry half for the
+// others. Each row sees the same products in the same order as if its
+// features had been copied and its empty segments filled with zeros, as an
+// earlier form did with a quarter of the gather warps' time (the fused kernel
+// of 4.19M camera rays 2.32 -> 2.03 ms, of a million secondary rays 1.41 ->
+// 1.27 ms). Gathers go round-robin over the gather warps in blocks of 32 items
+// (item = one point x one 16-byte column group), so every warp gets the same
+// share.
 //
 // Every mbarrier wait is bounded by a clock limit; on expiry the kernel flags
 // an abort, every role stops, the device error word is set, in-flight MMAs
@@ -42,6 +49,7 @@
 #include "device.cuh"
 #include "encode.cuh"
 #include "tc_common.cuh"
+#include "tile_feed.cuh"
 
 namespace lsnif {
 
@@ -57,15 +65,17 @@ __device__ __forceinline__ uint32_t idesc_f16(int N, int fp16) {
   return (1u << 4) | ab | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_f16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// off: rows (TMEM lanes) whose accumulators stay as they are
+__device__ __forceinline__ void mma_f16_rows(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, const uint4 &off,
+                                             uint32_t acc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n}\n" ::"r"(tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(off.x), "r"(off.y), "r"(off.z), "r"(off.w)
       : "memory");
 }
 
-// The same with the A operand read from tensor memory (a_tmem: lane 0 and
+// All rows, with the A operand read from tensor memory (a_tmem: lane 0 and
 // the first column of a 128-lane x K/2-column tile, row i in lane i, two
 // 16-bit values per column).
 __device__ __forceinline__ void mma_f16_ts(uint32_t tmem, uint32_t a_tmem, uint64_t b, uint32_t idesc, uint32_t acc) {
@@ -125,12 +135,12 @@ struct FusedArgs {
 // Shared-memory layout (byte offsets from a 1024-aligned base), the same on
 // host (sizing) and device (carving).
 struct Layout {
-  uint32_t blob, blob_lo, ring, ring_stride, ray, t0, t1, list, wsum, info, bars, tmem, misc, res, total;
+  uint32_t blob, blob_lo, ring, ring_stride, ray, list, masks, counts, info, bars, tmem, misc, res, total;
 };
 
 // mbarriers: full[kNBufMax], empty[kNBufMax], tile_ready[2], acc_full[2],
-// acc_empty[2], layer_done, fin[2]
-constexpr int kNumBars = 2 * kNBufMax + 2 + 2 + 2 + 1 + 2;
+// acc_empty[2], layer_done, fin[2], weights
+constexpr int kNumBars = 2 * kNBufMax + 2 + 2 + 2 + 1 + 2 + 1;
 
 // lo_bytes > 0 (BF16 operands): the later layers' residual weights, the lo
 // terms of their two-term products.
@@ -143,10 +153,9 @@ __host__ __device__ inline Layout make_layout(uint32_t blob_bytes, uint32_t lo_b
   o.blob_lo = lay_take(off, lo_bytes, 1024);
   o.ring = lay_take(off, (uint32_t)nbuf * o.ring_stride, 1024);
   o.ray = lay_take(off, 2 * kTileM * 4, 16);
-  o.t0 = lay_take(off, 2 * kTileM * 4, 16);
-  o.t1 = lay_take(off, 2 * kTileM * 4, 16);
   o.list = lay_take(off, 2u * (uint32_t)list_chunks * kListStride * 2u, 16);  // two tiles
-  o.wsum = lay_take(off, 2u * (uint32_t)list_chunks * 4u * 4u, 16);
+  o.masks = lay_take(off, 2u * (uint32_t)list_chunks * 4u * 8u, 16);
+  o.counts = lay_take(off, 2u * (uint32_t)list_chunks * 4u, 16);
   o.info = lay_take(off, 2 * sizeof(TileInfo), 16);
   o.bars = lay_take(off, 8 * kNumBars, 8);
   o.tmem = lay_take(off, 16, 16);
@@ -171,26 +180,33 @@ __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32
   TileInfo *s_info = reinterpret_cast<TileInfo *>(base + lay.info);
   uint64_t *bars = reinterpret_cast<uint64_t *>(base + lay.bars);
   uint64_t *b_full = bars, *b_empty = bars + kNBufMax, *b_ready = bars + 2 * kNBufMax;
-  uint64_t *b_accf = b_ready + 2, *b_acce = b_ready + 4, *b_fin = b_ready + 7;
+  uint64_t *b_accf = b_ready + 2, *b_acce = b_ready + 4, *b_fin = b_ready + 7, *b_w = b_ready + 9;
   int32_t *s_misc = reinterpret_cast<int32_t *>(base + lay.misc);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(s_misc + 4);
   const uint32_t ring_stride = lay.ring_stride;
   {
     // =================== MMA warp ===================
     int rbuf = 0, ruse = 0;  // ring slot and pass of the next chunk
+    int loads = 0;           // weight loads waited for
     const uint32_t idesc0 = idesc_f16(W, H16);
     for (int i = 0;; ++i) {
       const int tb = i & 1;
       if (!mbar_wait_sleep(su32(&b_ready[tb]), (uint32_t)((i >> 1) & 1), abort_flag)) break;
       const TileInfo ti = s_info[tb];
       if (ti.stop) break;
+      if (ti.loads != loads) {  // this tile is the first with its object's weights
+        loads = ti.loads;
+        if (!mbar_wait_sleep(su32(b_w), (uint32_t)((loads - 1) & 1), abort_flag)) break;
+      }
       const DevObject &ob = objs[ti.slot];
-      const int CHK = 2 * ob.L * F;
+      const int LF = ob.L * F, CHK = 2 * LF;
       const uint32_t a_sbo = (uint32_t)(CHK / 8) * 128u, w0_sbo = (uint32_t)(ob.n_in / 8) * 128u;
+      const uint4 *masks = reinterpret_cast<const uint4 *>(base + lay.masks) + (size_t)tb * a.list_chunks * 2;
       if (i >= 2 && !mbar_wait_sleep(su32(&b_acce[tb]), (uint32_t)(((i - 2) >> 1) & 1), abort_flag)) break;
       tc_after();
       const uint32_t dacc = tmem + (uint32_t)(tb * W);
       bool ok = true;
+      int prev = 0;  // ring slot of the chunk before
       for (int s = 0; s < ti.kmax; ++s) {
         // ring position of the next chunk, kept as counters (no division by
         // the run-time ring size)
@@ -206,14 +222,32 @@ __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32
         }
         tc_after();
         if (lane == 0) {
-          const uint32_t a0 = su32(s_ring + buf * ring_stride), b0 = su32(s_blob);
-          for (int ks = 0; ks < CHK / 16; ++ks) {
-            const uint64_t ad = umma_desc(a0 + ks * 256, 128, a_sbo);
-            const uint64_t bd = umma_desc(b0 + (uint32_t)((s * CHK) / 8 + 2 * ks) * 128u, 128, w0_sbo);
-            mma_f16(dacc, ad, bd, idesc0, (s > 0 || ks > 0) ? 1u : 0u);
+          const uint32_t a0 = su32(s_ring + buf * ring_stride), ap = su32(s_ring + prev * ring_stride),
+                         b0 = su32(s_blob) + (uint32_t)((s * CHK) / 8) * 128u;
+          // (rows with a segment s, of those the shared entry points) of warps 0, 1 | 2, 3
+          const uint4 m01 = masks[2 * s], m23 = masks[2 * s + 1];
+          const uint4 off = make_uint4(~m01.x, ~m01.z, ~m23.x, ~m23.z);
+          auto multiply = [&](uint32_t at, uint32_t bt, int steps, const uint4 &o, bool first) {
+            for (int ks = 0; ks < steps; ++ks)
+              mma_f16_rows(dacc, umma_desc(at + ks * 256, 128, a_sbo), umma_desc(bt + ks * 256, 128, w0_sbo), idesc0, o,
+                           first && ks == 0 ? 0u : 1u);
+          };
+          if (LF % 16 == 0) {
+            const int h = LF / 16;  // steps of one point
+            // entry points: the chunk before holds the shared ones as its exit points
+            if (m01.y | m01.w | m23.y | m23.w)
+              multiply(ap + h * 256, b0, h, make_uint4(~m01.y, ~m01.w, ~m23.y, ~m23.w), false);
+            multiply(a0, b0, h, make_uint4(off.x | m01.y, off.y | m01.w, off.z | m23.y, off.w | m23.w), s == 0);
+            multiply(a0 + h * 256, b0 + h * 256, h, off, false);
+          } else {
+            multiply(a0, b0, CHK / 16, off, s == 0);
           }
-          mma_commit(su32(&b_empty[buf]));
+          // the slot of the chunk before is free once these are done; the last
+          // chunk has no reader after it
+          if (s > 0) mma_commit(su32(&b_empty[prev]));
+          if (s + 1 == ti.kmax) mma_commit(su32(&b_empty[buf]));
         }
+        prev = buf;
         __syncwarp();
       }
       if (!ok) break;
@@ -233,7 +267,6 @@ __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32
 template <int F, int W, bool XROWS, int NG, bool H16>
 __device__ __noinline__ void epilogue_role(const FusedArgs *ap, uint8_t *base, uint32_t tmem) {
   const FusedArgs &a = *ap;
-  constexpr int fp16 = H16;
   constexpr int kEpiWarp0 = NG + 1;
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const QueryLaunch &q = a.q;
@@ -242,282 +275,168 @@ __device__ __noinline__ void epilogue_role(const FusedArgs *ap, uint8_t *base, u
   uint8_t *s_blob = base + lay.blob;
   uint8_t *s_blob_lo = base + lay.blob_lo;
   int32_t *s_ray = reinterpret_cast<int32_t *>(base + lay.ray);
-  float *s_t0 = reinterpret_cast<float *>(base + lay.t0);
-  float *s_t1 = reinterpret_cast<float *>(base + lay.t1);
   uint16_t *s_list = reinterpret_cast<uint16_t *>(base + lay.list);
-  uint32_t *s_wsum = reinterpret_cast<uint32_t *>(base + lay.wsum);
+  uint2 *s_masks = reinterpret_cast<uint2 *>(base + lay.masks);
+  int32_t *s_counts = reinterpret_cast<int32_t *>(base + lay.counts);
   TileInfo *s_info = reinterpret_cast<TileInfo *>(base + lay.info);
   uint64_t *bars = reinterpret_cast<uint64_t *>(base + lay.bars);
   uint64_t *b_ready = bars + 2 * kNBufMax;
   uint64_t *b_accf = b_ready + 2, *b_acce = b_ready + 4, *b_layer = b_ready + 6, *b_fin = b_ready + 7;
+  uint64_t *b_w = b_ready + 9;
   int32_t *s_misc = reinterpret_cast<int32_t *>(base + lay.misc);
   volatile int *abort_flag = reinterpret_cast<volatile int *>(s_misc + 4);
   float *s_res = reinterpret_cast<float *>(base + lay.res);
-  const int64_t n_tiles = XROWS ? (a.xrows + kTileM - 1) / kTileM : (int64_t)q.s.meta[1];
-  {
-    // =================== epilogue warps ===================
-    // Besides the layers after the first, these four warps set up every
-    // tile (fetch, rows, work lists, weights on an object change) one tile
-    // ahead, so the gather warps never stop between tiles.
-    constexpr int kEpiThreads = kEpiWarps * 32;
-    const int etid = tid - kEpiWarp0 * 32;  // 0..127: the row a setup thread handles
-    const int ew = etid >> 5;
-    const int quarter = warp & 3;           // the TMEM lane quarter this warp may access
-    const int r = quarter * 32 + lane;      // the row (ray) of the layers
-    const uint32_t act_sbo = (uint32_t)(W / 8) * 128u;
-    int layer_ctr = 0;
-    int su_slot = -1;  // object whose weights are in shared memory
+  // Besides the layers after the first, these four warps set up every tile
+  // (rows, work lists, weights on an object change) one tile ahead, so the
+  // gather warps never stop between tiles; the tile after that is fetched
+  // while the layers run.
+  const int etid = tid - kEpiWarp0 * 32;  // 0..127: the row a setup thread handles
+  const int quarter = warp & 3;           // the TMEM lane quarter this warp may access
+  const int r = quarter * 32 + lane;      // the row (ray) of the layers
+  const uint32_t act_sbo = (uint32_t)(W / 8) * 128u;
+  int layer_ctr = 0;
+  int su_slot = -1;  // object whose weights are in shared memory (or on their way)
+  int loads = 0;     // weight loads so far
+  TileFeed<XROWS> feed(q, abort_flag, s_misc, a.xrows, XROWS ? objs[0].H / 2 : 0, etid);
 
-    // next tile index (INT_MAX once aborted), uniform over the epilogue warps
-    auto fetch = [&]() -> int {
-      named_sync(2, kEpiThreads);
-      if (etid == 0) s_misc[0] = *abort_flag ? INT_MAX : atomicAdd(q.s.meta + 3, 1);
-      named_sync(2, kEpiThreads);
-      return s_misc[0];
-    };
-    auto slot_of_tile = [&](int tile) -> int { return XROWS ? 0 : q.s.tiles[3 * tile + 0]; };
-    // Set tile `tile` up as the j-th tile (slot j & 1). The slot's previous
-    // tile (j - 2) is finished by every role; a weight reload is only asked
-    // for once the previous tile's layers are done.
-    auto setup = [&](int j, int tile) {
-      const int sb = j & 1;
-      if ((int64_t)tile >= n_tiles) {
-        if (etid == 0) {
-          s_info[sb].stop = 1;
-          mbar_arrive(su32(&b_ready[sb]));
-        }
-        return;
-      }
-      int slot, start, cnt;
-      if (XROWS) {
-        slot = 0;
-        start = tile * kTileM;
-        cnt = (int)min((int64_t)kTileM, a.xrows - (int64_t)tile * kTileM);
-      } else {
-        slot = q.s.tiles[3 * tile + 0];
-        start = q.s.tiles[3 * tile + 1];
-        cnt = q.s.tiles[3 * tile + 2];
-      }
-      const DevObject &ob = objs[slot];
-      if (slot != su_slot) {
-        const uint4 *src = reinterpret_cast<const uint4 *>(H16 ? ob.umma_h : ob.umma);
-        uint4 *dst = reinterpret_cast<uint4 *>(s_blob);
-        const int nvec = (int)(ob.umma_bytes / 16);
-        for (int k = etid; k < nvec; k += kEpiThreads) dst[k] = __ldg(src + k);
-        if constexpr (!H16) {
-          const uint4 *src_lo = reinterpret_cast<const uint4 *>(ob.umma_lo);
-          uint4 *dst_lo = reinterpret_cast<uint4 *>(s_blob_lo);
-          const int nlo = (int)(ob.umma_lo_bytes / 16);
-          for (int k = etid; k < nlo; k += kEpiThreads) dst_lo[k] = __ldg(src_lo + k);
-        }
-        if (etid < LSNIF_MAX_LEVELS) s_res[etid] = (float)ob.res[etid];
-        fence_async_smem();
-        su_slot = slot;
-      }
-      if (etid == 0) s_misc[1] = 0;
-      named_sync(2, kEpiThreads);
-      // rows
-      int my_kk = 0;
-      uint32_t my_dm = 0u;
-      {
-        int ray = -1;
-        float t0v = 0.f, t1v = 0.f;
-        if (etid < cnt) {
-          if (XROWS) {
-            ray = start + etid;
-            my_kk = ob.H / 2;
-          } else {
-            ray = q.s.order[start + etid];
-            my_kk = q.s.k[ray];
-            my_dm = q.s.dup[ray];
-            const float2 tt = reinterpret_cast<const float2 *>(q.s.t01)[ray];
-            t0v = tt.x;
-            t1v = tt.y;
-          }
-        }
-        s_ray[sb * kTileM + etid] = ray;
-        s_t0[sb * kTileM + etid] = t0v;
-        s_t1[sb * kTileM + etid] = t1v;
-        const int wm = __reduce_max_sync(0xffffffffu, my_kk);
-        if (lane == 0) atomicMax(&s_misc[1], wm);
-      }
-      named_sync(2, kEpiThreads);
-      const int kmax = s_misc[1];
-      // work lists: per chunk, [gathers | copies | zero fills]
-      uint16_t *lst = s_list + (size_t)sb * a.list_chunks * kListStride;
-      uint32_t *ws = s_wsum + (size_t)sb * a.list_chunks * 4;
-      for (int s = 0; s < kmax; ++s) {
-        const uint32_t tot = __reduce_add_sync(0xffffffffu, row_counts(my_kk, my_dm, s));
-        if (lane == 0) ws[s * 4 + ew] = tot;
-      }
-      named_sync(2, kEpiThreads);
-      for (int s = 0; s < kmax; ++s) {
-        const uint32_t v = row_counts(my_kk, my_dm, s);
-        uint32_t incl = v;
-#pragma unroll
-        for (int o = 1; o < 32; o <<= 1) {
-          const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-          if (lane >= o) incl += y;
-        }
-        uint32_t woff = 0, all = 0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) {
-          const uint32_t x = ws[s * 4 + w];
-          all += x;
-          woff += w < ew ? x : 0u;
-        }
-        const uint32_t pos = incl - v + woff;
-        const int ngt = (int)(all & 1023u), nct = (int)((all >> 10) & 1023u);
-        uint16_t *Ls = lst + s * kListStride;
-        if (v & 1023u) {
-          const int pg = (int)(pos & 1023u);
-          if (v & (1023u << 10)) {  // entry point shared with the previous exit
-            Ls[pg] = (uint16_t)(etid | 128);
-            Ls[ngt + (int)((pos >> 10) & 1023u)] = (uint16_t)etid;
-          } else {
-            Ls[pg] = (uint16_t)etid;
-            Ls[pg + 1] = (uint16_t)(etid | 128);
-          }
-        } else {
-          const int pz = ngt + nct + (int)((pos >> 20) & 1023u);
-          Ls[pz] = (uint16_t)etid;
-          Ls[pz + 1] = (uint16_t)(etid | 128);
-        }
-      }
-      named_sync(2, kEpiThreads);
+  // Set the fetched tile up as the j-th (slot j & 1). The slot's previous
+  // tile (j - 2) is finished by every role; a weight reload is only asked
+  // for once the previous tile's layers are done.
+  auto setup = [&](int j) {
+    const int sb = j & 1;
+    if (feed.cnt < 0) {
       if (etid == 0) {
-        s_info[sb].kmax = kmax;
-        s_info[sb].slot = slot;
-        s_info[sb].stop = 0;
+        s_info[sb].stop = 1;
         mbar_arrive(su32(&b_ready[sb]));
       }
-    };
-
-    int stop_at = INT_MAX;
-    {
-      const int t0i = fetch();
-      setup(0, t0i);
-      if ((int64_t)t0i >= n_tiles) stop_at = 0;
+      return;
     }
-    for (int i = 0; i < stop_at; ++i) {
-      const int tb = i & 1;
-      // set up tile i+1 now, unless it needs other weights: then after the
-      // layers of tile i, which still read the current ones
-      const int tn = fetch();
-      const bool last = (int64_t)tn >= n_tiles;
-      const bool deferred = !last && slot_of_tile(tn) != su_slot;
-      if (!deferred) setup(i + 1, tn);
-      if (last) stop_at = i + 1;
+    if (feed.slot != su_slot) {
+      const DevObject &ob = objs[feed.slot];
+      ++loads;
+      su_slot = feed.slot;
+      if (etid == 0) {
+        // two bulk copies; whoever needs the weights waits for their barrier,
+        // the gathers start without them (16-byte loads by these warps held
+        // the first tile up by about 5 us)
+        fence_async_smem();
+        const uint32_t lo = H16 ? 0u : ob.umma_lo_bytes;
+        mbar_expect(su32(b_w), ob.umma_bytes + lo);
+        bulk_load(su32(s_blob), H16 ? ob.umma_h : ob.umma, ob.umma_bytes, su32(b_w));
+        if (lo) bulk_load(su32(s_blob_lo), ob.umma_lo, lo, su32(b_w));
+      }
+      if (etid < LSNIF_MAX_LEVELS) s_res[etid] = (float)ob.res[etid];
+    }
+    s_ray[sb * kTileM + etid] = feed.ray;
+    // a half step of K (L F = 8 mod 16) cannot be read from another chunk's
+    // tile: shared points are gathered twice then
+    const uint32_t dm = (objs[feed.slot].L * F) % 16 == 0 ? feed.dm : 0u;
+    const int kmax = build_lists<false>(etid, feed.kk, dm, s_list + (size_t)sb * a.list_chunks * kListStride,
+                                        s_masks + (size_t)sb * a.list_chunks * 4,
+                                        s_counts + (size_t)sb * a.list_chunks, s_misc, a.list_chunks);
+    named_sync(2, kFeedThreads);
+    if (etid == 0) {
+      s_info[sb].kmax = kmax;
+      s_info[sb].slot = feed.slot;
+      s_info[sb].stop = 0;
+      s_info[sb].rows = (int16_t)feed.cnt;
+      s_info[sb].loads = (int16_t)(loads & 0x7fff);
+      mbar_arrive(su32(&b_ready[sb]));
+    }
+    feed.stage = 0;
+  };
 
-      // ---- layers after the first, decode ----
-      if (etid == 0) s_misc[2] = mbar_wait_sleep(su32(&b_accf[tb]), (uint32_t)((i >> 1) & 1), abort_flag) ? 0 : 1;
-      named_sync(2, kEpiThreads);
-      if (!s_misc[2]) {
-        tc_after();
-        const TileInfo ti = s_info[tb];
-        const DevObject &ob = objs[ti.slot];
-        const int n_hidden = ob.n_hidden, n_out = ob.n_out, n_out_pad = ob.n_out_pad, n_mat = ob.n_mat,
-                  act = ob.act;
-        const float *bias = reinterpret_cast<const float *>(s_blob + ob.umma_bias_off);
-        const uint32_t wl_off0 = (uint32_t)W * ob.n_in * 2u;  // byte offset of W1 in the blob
-        uint32_t wl_off = wl_off0;
-        const uint32_t dacc = tmem + (uint32_t)(tb * W);
-        const uint32_t trow = dacc + ((uint32_t)(quarter * 32) << 16);
-        const uint32_t act_col = tmem + (uint32_t)(2 * W);  // activation tile (A operand), lane 0
-        const uint32_t tact = act_col + ((uint32_t)(quarter * 32) << 16), tact_lo = tact + (uint32_t)(W / 2);
-        for (int layer = 0; layer <= n_hidden; ++layer) {
-          const bool out_layer = layer == n_hidden;
-          const float *bl = bias + layer * W;
-          if (!out_layer) {
-            const int N = (layer + 1 < n_hidden) ? W : n_out_pad;
-            const uint32_t idesc = idesc_f16(N, fp16);
-            // The activations go to tensor memory, row r in lane r, two 16-bit
-            // values per 32-bit column (the A operand of tcgen05.mma read from
-            // TMEM): hi at columns [2W, 2W + W/2), lo (two-term BF16) after it.
-#pragma unroll
-            for (int c0 = 0; c0 < W; c0 += 16) {
-              uint32_t v[16];
-              TMEM_LD16(trow + c0, (&v[0]));
-              tmem_wait_ld();
-              uint32_t hw[8];
-              if constexpr (H16) {
-#pragma unroll
-                for (int u = 0; u < 8; ++u)
-                  hw[u] = pack_op(act_fn(__uint_as_float(v[2 * u]) + bl[c0 + 2 * u], act),
-                                  act_fn(__uint_as_float(v[2 * u + 1]) + bl[c0 + 2 * u + 1], act), fp16);
-              } else {
-                // two-term BF16: hi = BF16(h), lo = BF16(h - hi) (the difference is exact in FP32)
-                uint32_t lw[8];
-#pragma unroll
-                for (int u = 0; u < 8; ++u) {
-                  const float x0 = act_fn(__uint_as_float(v[2 * u]) + bl[c0 + 2 * u], act);
-                  const float x1 = act_fn(__uint_as_float(v[2 * u + 1]) + bl[c0 + 2 * u + 1], act);
-                  const __nv_bfloat162 hb = __floats2bfloat162_rn(x0, x1);
-                  const float2 hf = __bfloat1622float2(hb);
-                  hw[u] = *reinterpret_cast<const uint32_t *>(&hb);
-                  lw[u] = pack_bf16(x0 - hf.x, x1 - hf.y);
-                }
-                TMEM_ST8(tact_lo + (uint32_t)(c0 / 2), lw);
-              }
-              TMEM_ST8(tact + (uint32_t)(c0 / 2), hw);
-            }
-            tmem_wait_st();
-            tc_before();
-            named_sync(2, kEpiThreads);
-            if (etid == 0) {
-              tc_after();
-              const uint32_t b0 = su32(s_blob) + wl_off, b0l = su32(s_blob_lo) + (wl_off - wl_off0);
-              for (int ks = 0; ks < W / 16; ++ks) {
-                const uint64_t bd = umma_desc(b0 + ks * 256, 128, act_sbo);
-                mma_f16_ts(dacc, act_col + (uint32_t)(ks * 8), bd, idesc, ks > 0 ? 1u : 0u);
-                if constexpr (!H16) {
-                  // the lo terms: hi_a . lo_w + lo_a . hi_w (lo_a . lo_w is left out)
-                  mma_f16_ts(dacc, act_col + (uint32_t)(ks * 8), umma_desc(b0l + ks * 256, 128, act_sbo), idesc, 1u);
-                  mma_f16_ts(dacc, act_col + (uint32_t)(W / 2 + ks * 8), bd, idesc, 1u);
-                }
-              }
-              mma_commit(su32(b_layer));
-              mbar_wait_sleep(su32(b_layer), (uint32_t)(layer_ctr & 1), abort_flag);
-            }
-            ++layer_ctr;
-            named_sync(2, kEpiThreads);
-            tc_after();
-            wl_off += (uint32_t)N * W * 2u;
-          } else {
-            // logits 16 columns at a time into a per-thread array, then decode
-            float z[64];
-#pragma unroll 1
-            for (int c0 = 0; c0 < n_out_pad; c0 += 16) {
-              uint32_t v[16];
-              TMEM_LD16(trow + c0, (&v[0]));
-              tmem_wait_ld();
-#pragma unroll
-              for (int u = 0; u < 16; ++u) z[c0 + u] = __uint_as_float(v[u]) + bl[c0 + u];
-            }
-            const int32_t ray = s_ray[tb * kTileM + r];
-            if (ray >= 0 && !*abort_flag) {
-              if (XROWS) {
-                for (int j = 0; j < n_out; ++j) a.Z[(int64_t)ray * n_out + j] = z[j];
-              } else {
-                decode_store(q.hits, ray, z, n_out, n_mat, s_t0[tb * kTileM + r], s_t1[tb * kTileM + r],
-                             q.rays.tmin[ray], q.rays.tmax[ray]);
-              }
+  feed.finish();
+  int stop_at = feed.cnt < 0 ? 0 : INT_MAX;
+  setup(0);
+  for (int i = 0; i < stop_at; ++i) {
+    const int tb = i & 1;
+    // set up tile i+1 now, unless it needs other weights: then after the
+    // layers of tile i, which still read the current ones
+    feed.finish();
+    const bool last = feed.cnt < 0, deferred = !last && feed.slot != su_slot;
+    if (!deferred) setup(i + 1);
+    if (last) stop_at = i + 1;
+
+    // ---- layers after the first, decode ----
+    if (etid == 0) {
+      // the accumulator, and with it the weights, which its MMAs have read
+      const bool got = mbar_wait(su32(&b_accf[tb]), (uint32_t)((i >> 1) & 1), abort_flag) &&
+                       mbar_wait(su32(b_w), (uint32_t)((s_info[tb].loads - 1) & 1), abort_flag);
+      s_misc[2] = got ? 0 : 1;
+    }
+    named_sync(2, kFeedThreads);
+    if (!s_misc[2]) {
+      tc_after();
+      const DevObject &ob = objs[s_info[tb].slot];
+      const int n_hidden = ob.n_hidden, n_out_pad = ob.n_out_pad;
+      const bool relu = ob.act == 0;
+      const float *bias = reinterpret_cast<const float *>(s_blob + ob.umma_bias_off);
+      const uint32_t wl_off0 = (uint32_t)W * ob.n_in * 2u;  // byte offset of W1 in the blob
+      uint32_t wl_off = wl_off0;
+      const uint32_t dacc = tmem + (uint32_t)(tb * W);
+      const uint32_t trow = dacc + ((uint32_t)(quarter * 32) << 16);
+      const uint32_t act_col = tmem + (uint32_t)(2 * W);  // activation tile (A operand), lane 0
+      const uint32_t tact = act_col + ((uint32_t)(quarter * 32) << 16), tact_lo = tact + (uint32_t)(W / 2);
+      const int ray = s_ray[tb * kTileM + r];
+      float tmin = 0.f, tmax = 0.f;
+      float2 t01 = make_float2(0.f, 0.f);
+      for (int layer = 0; layer < n_hidden; ++layer) {
+        const float *bl = bias + layer * W;
+        const int N = (layer + 1 < n_hidden) ? W : n_out_pad;
+        const uint32_t idesc = idesc_f16(N, H16);
+        // The activations go to tensor memory, row r in lane r, two 16-bit
+        // values per 32-bit column (the A operand of tcgen05.mma read from
+        // TMEM): hi at columns [2W, 2W + W/2), lo (two-term BF16) after it.
+        if (relu) layer_activations<W, H16, true>(trow, tact, tact_lo, bl);
+        else layer_activations<W, H16, false>(trow, tact, tact_lo, bl);
+        tmem_wait_st();
+        tc_before();
+        named_sync(2, kFeedThreads);
+        if (etid == 0) {
+          tc_after();
+          const uint32_t b0 = su32(s_blob) + wl_off, b0l = su32(s_blob_lo) + (wl_off - wl_off0);
+          for (int ks = 0; ks < W / 16; ++ks) {
+            const uint64_t bd = umma_desc(b0 + ks * 256, 128, act_sbo);
+            mma_f16_ts(dacc, act_col + (uint32_t)(ks * 8), bd, idesc, ks > 0 ? 1u : 0u);
+            if constexpr (!H16) {
+              // the lo terms: hi_a . lo_w + lo_a . hi_w (lo_a . lo_w is left out)
+              mma_f16_ts(dacc, act_col + (uint32_t)(ks * 8), umma_desc(b0l + ks * 256, 128, act_sbo), idesc, 1u);
+              mma_f16_ts(dacc, act_col + (uint32_t)(W / 2 + ks * 8), bd, idesc, 1u);
             }
           }
+          mma_commit(su32(b_layer));
         }
+        // while the MMAs run: the next tile but one, and the decode's inputs
+        if (!deferred && !last && feed.stage < 5) feed.step();
+        if (!XROWS && layer + 1 == n_hidden && ray >= 0) {
+          tmin = q.rays.tmin[ray];
+          tmax = q.rays.tmax[ray];
+          t01 = reinterpret_cast<const float2 *>(q.s.t01)[ray];
+        }
+        if (etid == 0) mbar_wait(su32(b_layer), (uint32_t)(layer_ctr & 1), abort_flag);
+        ++layer_ctr;
+        named_sync(2, kFeedThreads);
+        tc_after();
+        wl_off += (uint32_t)N * W * 2u;
       }
-      tc_before();
-      mbar_arrive(su32(&b_acce[tb]));
-      if (deferred) {
-        named_sync(2, kEpiThreads);  // every thread is done with the old weights
-        setup(i + 1, tn);
-      }
+      store_outputs<XROWS>(q.hits, a.Z, trow, bias + n_hidden * W, ray, ray >= 0 && !*abort_flag, ob.n_out, n_out_pad,
+                           ob.n_mat, t01.x, t01.y, tmin, tmax);
     }
-    if (etid == 0) {
-      mma_commit(su32(&b_fin[1]));
-      if (!mbar_wait_teardown(su32(&b_fin[1]), 0u)) *abort_flag = 1;
+    tc_before();
+    mbar_arrive(su32(&b_acce[tb]));
+    if (deferred) {
+      named_sync(2, kFeedThreads);  // every thread is done with the old weights
+      setup(i + 1);
     }
-    }
+  }
+  if (etid == 0) {
+    // a weight copy still in flight (after an abort) lands before the shared
+    // memory is released
+    if (loads > 0 && !mbar_wait_teardown(su32(b_w), (uint32_t)((loads - 1) & 1))) *abort_flag = 1;
+    mma_commit(su32(&b_fin[1]));
+    if (!mbar_wait_teardown(su32(&b_fin[1]), 0u)) *abort_flag = 1;
+  }
 }
 
 // F: features per level; W: hidden width; XROWS: read the network input
@@ -543,11 +462,12 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
   uint8_t *s_ring = base + lay.ring;
   int32_t *s_ray = reinterpret_cast<int32_t *>(base + lay.ray);
   uint16_t *s_list = reinterpret_cast<uint16_t *>(base + lay.list);
-  uint32_t *s_wsum = reinterpret_cast<uint32_t *>(base + lay.wsum);
+  const int32_t *s_counts = reinterpret_cast<const int32_t *>(base + lay.counts);
   TileInfo *s_info = reinterpret_cast<TileInfo *>(base + lay.info);
   uint64_t *bars = reinterpret_cast<uint64_t *>(base + lay.bars);
   uint64_t *b_full = bars, *b_empty = bars + kNBufMax, *b_ready = bars + 2 * kNBufMax;
   uint64_t *b_accf = b_ready + 2, *b_acce = b_ready + 4, *b_layer = b_ready + 6, *b_fin = b_ready + 7;
+  uint64_t *b_w = b_ready + 9;
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(base + lay.tmem);
   int32_t *s_misc = reinterpret_cast<int32_t *>(base + lay.misc);  // [0] tile [1] kmax [2] epi stop [4] abort
   volatile int *abort_flag = reinterpret_cast<volatile int *>(s_misc + 4);
@@ -566,6 +486,9 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
       mbar_init(su32(&b_fin[b]), 1);
     }
     mbar_init(su32(b_layer), 1);
+    mbar_init(su32(b_w), 1);
+    // make the initialised barriers visible to the bulk-copy unit
+    asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
     *abort_flag = 0;
   }
   if (warp == 0) {
@@ -587,7 +510,7 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
     uint32_t mask = 0;
     const uint16_t *tab = nullptr;
     int rbuf = 0, ruse = 0;    // ring slot and pass of the next chunk
-    int rot_g = 0, rot_o = 0;  // round-robin origin of the gather / other blocks
+    int rot_g = 0;             // round-robin origin of the gather blocks
     for (int i = 0;; ++i) {
       const int tb = i & 1;
       // the epilogue warps set the tile up: rows, work lists, weights
@@ -604,7 +527,7 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
         cur_slot = ti.slot;
       }
       const uint16_t *s_lst = s_list + (size_t)tb * a.list_chunks * kListStride;
-      const uint32_t *s_ws = s_wsum + (size_t)tb * a.list_chunks * 4;
+      const int32_t *s_cnt = s_counts + (size_t)tb * a.list_chunks;
 
       // ---- chunks ----
       const int G = (L * F) / 8;  // 16-byte column groups per point
@@ -636,25 +559,13 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
           rbuf = 0;
           ++ruse;
         }
-        // chunk c - 1 (whose exit points the copies read) and chunk
-        // c - nbuf + 1 (which read this slot's previous chunk)
-        const int pbuf = buf > 0 ? buf - 1 : nbuf - 1, puse = buf > 0 ? use : use - 1;
-        const bool wrap = buf + 1 == nbuf;
-        const int nbuf1 = wrap ? 0 : buf + 1, nuse1 = wrap ? use : use - 1;
         uint8_t *A = s_ring + buf * ring_stride;
-        uint32_t all = 0;
-#pragma unroll
-        for (int w = 0; w < 4; ++w) all += s_ws[s * 4 + w];
-        const int ngt = (int)(all & 1023u), nct = (int)((all >> 10) & 1023u);
-        const int n_gi = ngt * G, n_oi = (kListStride - ngt) * G;
-        const int nb_g = (n_gi + 31) >> 5, nb_o = (n_oi + 31) >> 5;
-        const int first_g = (warp - rot_g + NG) % NG, first_o = (warp - rot_o + NG) % NG;
-        // The buffer is free once the MMAs of chunk c - nbuf are done and the
-        // copies of chunk c - nbuf + 1 (which read it) are written. Every
-        // thread waits, with or without items: an arrival on the full barrier
-        // must not land in the phase of chunk c - nbuf.
+        const int ngt = s_cnt[s], n_gi = ngt * G, nb_g = (n_gi + 31) >> 5;
+        const int first_g = (warp - rot_g + NG) % NG;
+        // the slot is free once the MMAs that read its last chunk are done.
+        // Every thread waits, with or without items: an arrival on the full
+        // barrier must not land in the phase of that chunk.
         if (use > 0) mbar_wait_sleep(su32(&b_empty[buf]), (uint32_t)((use - 1) & 1), abort_flag);
-        if (nbuf > 1 && nuse1 >= 0) mbar_wait_sleep(su32(&b_full[nbuf1]), (uint32_t)(nuse1 & 1), abort_flag);
         // gathers: the lanes of a warp take consecutive entries (neighbouring
         // rays) at the same column group, so at coarse levels they share
         // corners and cache sectors
@@ -670,10 +581,7 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
               if (bn * 32 + lane < n_gi) pn = load_point(s, bn * 32 + lane, ngt, inv_g);
             } else if (s + 1 < kmax) {
               // this thread's first item of the next chunk
-              uint32_t all2 = 0;
-#pragma unroll
-              for (int w = 0; w < 4; ++w) all2 += s_ws[(s + 1) * 4 + w];
-              const int ngt2 = (int)(all2 & 1023u), n_gi2 = ngt2 * G;
+              const int ngt2 = s_cnt[s + 1], n_gi2 = ngt2 * G;
               const int first2 = (warp - (rot_g + nb_g) % NG + NG) % NG;
               if (first2 * 32 + lane < n_gi2) {
                 pn = load_point(s + 1, first2 * 32 + lane, ngt2, 1.f / (float)max(ngt2, 1));
@@ -740,28 +648,7 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
             *reinterpret_cast<uint4 *>(A + core_off(r, j * G + g, a_sbo)) = outv;
           }
         }
-        // copies (entry point = previous chunk's exit point) and zero fills
-        const int n_o = kListStride - ngt;
-        if (nct > 0 && first_o < nb_o)  // copies read the previous chunk: it must be complete
-          mbar_wait_sleep(su32(&b_full[pbuf]), (uint32_t)(puse & 1), abort_flag);
-        const float inv_o = 1.f / (float)max(n_o, 1);
-        for (int b = first_o; b < nb_o; b += NG) {
-          const int it = b * 32 + lane;
-          if (it < n_oi) {
-            const int g = __float2int_rz(((float)it + 0.5f) * inv_o);
-            const int t = it - g * n_o;
-            const int e = s_lst[s * kListStride + ngt + t];
-            const int r = e & 127, j = e >> 7;
-            uint4 outv = make_uint4(0u, 0u, 0u, 0u);
-            if (t < nct) {
-              const uint8_t *Ap = s_ring + pbuf * ring_stride;
-              outv = *reinterpret_cast<const uint4 *>(Ap + core_off(r, G + g, a_sbo));
-            }
-            *reinterpret_cast<uint4 *>(A + core_off(r, j * G + g, a_sbo)) = outv;
-          }
-        }
         rot_g = (rot_g + nb_g) % NG;
-        rot_o = (rot_o + nb_o) % NG;
         fence_async_smem();
         mbar_arrive(su32(&b_full[buf]));
       }
@@ -834,7 +721,7 @@ static cudaError_t launch_op(const FusedArgs &a, size_t smem, cudaStream_t st) {
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // one persistent CTA per SM, but no more CTAs than the batch can have
   // tiles: a small request leaves the other SMs to concurrent work
-  const int64_t tiles = XR ? (a.xrows + kTileM - 1) / kTileM : (int64_t)a.q.s.max_tiles;
+  const int64_t tiles = XR ? (a.xrows + kTileM - 1) / kTileM : fused_items_max(a.q);
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, tiles));
   fused_kernel<F, W, XR, NG, NLB, GS, H16><<<grid, (NG + 1 + kEpiWarps) * 32, smem, st>>>(a);
   return cudaGetLastError();

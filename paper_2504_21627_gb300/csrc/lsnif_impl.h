@@ -17,6 +17,7 @@ constexpr uint32_t kPi3 = 805459861u;
 constexpr int kMaxCap = 32;          // H/2 <= 32
 constexpr int kMaxObjects = 1024;    // object slots of a context
 constexpr int kMetaWords = 64;       // words of QueryScratch::meta
+constexpr int kMetaShift = 5;        // meta word: log2 of the parts a tile is worked on in
 constexpr int kBuckets = kMaxCap + 1;  // per object: k = 0..32
 constexpr int kTileM = 128;          // rays per tensor-core tile (tcgen05 M)
 constexpr int kDistCap = 32;         // largest stored occupancy distance
@@ -128,7 +129,7 @@ struct QueryScratch {
   int32_t *offsets;  // n_slots x kBuckets
   int32_t *cursor;   // n_slots x kBuckets
   int32_t *tiles;    // max_tiles x 3 (slot, start, count)
-  int32_t *meta;     // [0] n_live, [1] n_tiles, [2] n_points, [3] tile cursor
+  int32_t *meta;     // [0] n_live, [1] n_tiles, [2] n_points, [3] tile cursor, [4] ray counter, [5] kMetaShift
   float *X;          // FP32 path: chunk of tiles x kTileM rows x ldx features
   int32_t *blk;      // coherent grouping: live rays and points per block of kGroupBlock rays, then offsets
   int32_t *bins;     // counting sorts: rays per bin, then each bin's first position (kBinsAlloc)
@@ -145,6 +146,7 @@ struct QueryLaunch {
   HitsArg hits;
   QueryScratch s;
   int *err;               // device error word
+  int sms;                // the device's SMs
   cudaStream_t stream;
   int trace_mode;         // traversal kernel: 0 one ray per thread, 1 persistent lanes, 2 persistent lanes
                           // over rays presorted by (object, entry cell, direction octant)

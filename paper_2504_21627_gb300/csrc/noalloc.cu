@@ -154,6 +154,7 @@ extern "C" int lsnif_query_rays_noalloc(lsnif_ctx *ctx, const lsnif_rays *r, lsn
   q.hits = HitsArg{h->hit, h->t, h->nx, h->ny, h->nz, h->mat, h->ar, h->ag, h->ab, h->logits};
   q.s = s;
   q.err = ctx->d_err;
+  q.sms = ctx->sms;
   q.stream = (cudaStream_t)stream;
   q.trace_mode = ctx->trace_mode;
   q.group_mode = ctx->group_mode == 2 ? 3 : ctx->group_mode == 1 ? (r->obj ? 2 : 1) : 0;

@@ -508,6 +508,22 @@ __device__ __forceinline__ int block_scan(int v, int *ws, int &total) {
   return before;
 }
 
+// Parts (log2) in which the 16-bit fused kernels work on each tile: 1, 2 or
+// 4 of 128, 64 or 32 rows. Their time is a start plus a term per round of the
+// chip (the SM with the most parts), and smaller parts have shorter starts and
+// rounds but more of them. Measured on the torus network (16 levels), in us:
+// 128 rows 35 + 55 per round, 64 rows 25 + 28.5, 32 rows 22 + 17.5 -- so 3,000
+// rays take 39 us in 32-row parts and 88 in whole tiles, 20,000 rays 57 in
+// 64-row parts and 80 in whole tiles. On the icosphere network (8 levels),
+// where the layers weigh more, a smaller part gains less: it has to win by a
+// tenth.
+__device__ __forceinline__ int tile_shift(int n_live, int sms) {
+  auto rounds = [&](int rows) { return (n_live + rows * sms - 1) / (rows * sms); };
+  if (rounds(128) > 4) return 0;
+  const int c0 = 350 + 550 * rounds(128), c1 = 275 + 313 * rounds(64), c2 = 242 + 192 * rounds(32);
+  return c2 < c1 && c2 < c0 ? 2 : (c1 < c0 ? 1 : 0);
+}
+
 // Single block: bucket offsets (object ascending, k descending), tiles of
 // kTileM rays that never straddle objects, totals, cursors reset. A warp takes
 // one object's 32 buckets at a time, so an object's range starts at the value
@@ -553,6 +569,7 @@ __global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
     q.s.meta[1] = tiles;
     q.s.meta[2] = points;
     q.s.meta[3] = 0;
+    q.s.meta[kMetaShift] = tile_shift(run, q.sms);
   }
   __syncthreads();
   for (int t = threadIdx.x; t < tiles; t += blockDim.x) {
@@ -689,6 +706,7 @@ __global__ void __launch_bounds__(1024) group_scan_kernel(QueryLaunch q, int nbl
     q.s.meta[1] = tiles;
     q.s.meta[2] = points;
     q.s.meta[3] = 0;
+    q.s.meta[kMetaShift] = tile_shift(n_live, q.sms);
   }
   for (int b = b0; b < min(b0 + per, nblk); ++b) {   // block offsets replace the counts
     const int v = q.s.blk[b];

@@ -234,6 +234,7 @@ int lsnif::run_query(lsnif_ctx *ctx, Workspace *ws, const lsnif_rays *r, lsnif_h
   q.s = carve(ws, r->n, sh.H, sh.n_slots, n_in);
   q.s.wmax = sh.wmax;
   q.err = err;
+  q.sms = ctx->sms;
   q.stream = st;
   q.trace_mode = ctx->trace_mode;
   q.group_mode = ctx->group_mode == 2 ? 3 : ctx->group_mode == 1 ? (r->obj ? 2 : 1) : 0;

@@ -3,6 +3,7 @@
 // no-swizzle K-major core-matrix layout and the per-tile work-list rule.
 #pragma once
 
+#include <algorithm>
 #include <cstdint>
 
 #include "lsnif_impl.h"
@@ -118,6 +119,18 @@ __device__ __forceinline__ void tmem_wait_ld() { asm volatile("tcgen05.wait::ld.
 
 __device__ __forceinline__ void tmem_wait_st() { asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory"); }
 
+// 1-D bulk copies global -> shared completing on an mbarrier (addresses and
+// sizes multiples of 16 bytes): one expect of the sum, then the copies
+__device__ __forceinline__ void mbar_expect(uint32_t mbar, uint32_t bytes) {
+  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
+}
+
+__device__ __forceinline__ void bulk_load(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
+  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
+               "l"(src), "r"(bytes), "r"(mbar)
+               : "memory");
+}
+
 // byte offset of the 16-byte row piece (row r, core K-group kg of 16 bytes)
 // in a tile of 8-row core matrices with row-group stride sbo
 __device__ __forceinline__ uint32_t core_off(int r, int kg, uint32_t sbo) {
@@ -125,7 +138,9 @@ __device__ __forceinline__ uint32_t core_off(int r, int kg, uint32_t sbo) {
 }
 
 struct TileInfo {
-  int32_t kmax, slot, stop, pad;
+  int32_t kmax, slot, stop;
+  int16_t rows;   // rows of the tile
+  int16_t loads;  // weight loads up to this tile (low 15 bits)
 };
 
 __host__ __device__ inline uint32_t lay_take(uint32_t &off, uint32_t bytes, uint32_t align) {
@@ -133,6 +148,12 @@ __host__ __device__ inline uint32_t lay_take(uint32_t &off, uint32_t bytes, uint
   const uint32_t r = off;
   off += bytes;
   return r;
+}
+
+// Most work items a query's tiles are cut into (32 rows each, or whole
+// tiles): the widest grid that is of use.
+inline int64_t fused_items_max(const QueryLaunch &q) {
+  return std::max<int64_t>(q.s.max_tiles, std::min<int64_t>(q.rays.n / 32 + q.n_slots + 1, q.sms));
 }
 
 // work-list counts of one ray for chunk s, packed: gathers | copies << 10 |
