@@ -21,6 +21,7 @@
 #include "device.cuh"
 #include "encode.cuh"
 #include "tc_common.cuh"
+#include "tile_feed.cuh"
 
 namespace lsnif {
 
@@ -34,11 +35,13 @@ __device__ __forceinline__ uint32_t idesc_h16(int N) {
   return (1u << 4) | ((uint32_t)(N >> 3) << 17) | ((uint32_t)(kTileM >> 4) << 24);
 }
 
-__device__ __forceinline__ void mma_h16(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, uint32_t acc) {
+// off: rows (TMEM lanes) whose accumulators stay as they are
+__device__ __forceinline__ void mma_h16_rows(uint32_t tmem, uint64_t a, uint64_t b, uint32_t idesc, const uint4 &off,
+                                             uint32_t acc) {
   asm volatile(
       "{\n.reg .pred p;\nsetp.ne.b32 p, %4, 0;\n"
-      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, p;\n}\n" ::"r"(tmem),
-      "l"(a), "l"(b), "r"(idesc), "r"(acc)
+      "tcgen05.mma.cta_group::1.kind::f16 [%0], %1, %2, %3, {%5, %6, %7, %8}, p;\n}\n" ::"r"(tmem),
+      "l"(a), "l"(b), "r"(idesc), "r"(acc), "r"(off.x), "r"(off.y), "r"(off.z), "r"(off.w)
       : "memory");
 }
 
@@ -59,13 +62,10 @@ __device__ __forceinline__ uint32_t h2_sat(float a, float b) {
   return *reinterpret_cast<uint32_t *>(&v);
 }
 
-// 1-D bulk copy global -> shared completing on an mbarrier (both addresses
-// and the size multiples of 16 bytes)
+// one bulk copy (both addresses and the size multiples of 16 bytes)
 __device__ __forceinline__ void bulk_copy(uint32_t dst, const void *src, uint32_t bytes, uint32_t mbar) {
-  asm volatile("mbarrier.arrive.expect_tx.shared::cta.b64 _, [%0], %1;" ::"r"(mbar), "r"(bytes) : "memory");
-  asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(dst),
-               "l"(src), "r"(bytes), "r"(mbar)
-               : "memory");
+  mbar_expect(mbar, bytes);
+  bulk_load(dst, src, bytes, mbar);
 }
 
 __host__ __device__ constexpr int tmem_cols16s(int W) { return 3 * W <= 256 ? 256 : 512; }
@@ -80,7 +80,7 @@ struct Fused16sArgs {
 // W x CHK] (16-bit, CHK = 2 x 16 x F columns at most), the layer buffer
 // (W x W 16-bit weights), the biases, then the per-tile state.
 struct Layout16s {
-  uint32_t ring, slot_w, ring_stride, lbuf, bias, ray, t0, t1, list, wsum, info, bars, tmem, misc, res, total;
+  uint32_t ring, slot_w, ring_stride, lbuf, bias, ray, list, masks, counts, info, bars, tmem, misc, res, total;
 };
 
 // mbarriers: full[2], empty[2], wfull[2] (a slot's first-layer slice
@@ -98,10 +98,9 @@ __host__ __device__ inline Layout16s make_layout16s(int F, int W, int list_chunk
   o.lbuf = lay_take(off, (uint32_t)W * W * 2u, 1024);
   o.bias = lay_take(off, (uint32_t)max_bias * 4u, 16);
   o.ray = lay_take(off, 2 * kTileM * 4, 16);
-  o.t0 = lay_take(off, 2 * kTileM * 4, 16);
-  o.t1 = lay_take(off, 2 * kTileM * 4, 16);
   o.list = lay_take(off, 2u * (uint32_t)list_chunks * kListStride * 2u, 16);
-  o.wsum = lay_take(off, 2u * (uint32_t)list_chunks * 4u * 4u, 16);
+  o.masks = lay_take(off, 2u * (uint32_t)list_chunks * 4u * 8u, 16);
+  o.counts = lay_take(off, 2u * (uint32_t)list_chunks * 4u, 16);
   o.info = lay_take(off, 2 * sizeof(TileInfo), 16);
   o.bars = lay_take(off, 8 * kNumBars16s, 8);
   o.tmem = lay_take(off, 16, 16);
@@ -115,9 +114,9 @@ struct Smem16s {
   uint8_t *ring, *lbuf;
   float *bias;
   int32_t *ray;
-  float *t0, *t1;
   uint16_t *list;
-  uint32_t *wsum;
+  uint2 *masks;
+  int32_t *counts;
   TileInfo *info;
   uint64_t *full, *empty, *wfull, *ready, *accf, *acce, *layer, *lwfull, *fin;
   uint32_t *tmem;
@@ -135,10 +134,9 @@ __device__ __forceinline__ Smem16s carve16s(const Fused16sArgs &a, uint8_t *base
   S.lbuf = base + l.lbuf;
   S.bias = reinterpret_cast<float *>(base + l.bias);
   S.ray = reinterpret_cast<int32_t *>(base + l.ray);
-  S.t0 = reinterpret_cast<float *>(base + l.t0);
-  S.t1 = reinterpret_cast<float *>(base + l.t1);
   S.list = reinterpret_cast<uint16_t *>(base + l.list);
-  S.wsum = reinterpret_cast<uint32_t *>(base + l.wsum);
+  S.masks = reinterpret_cast<uint2 *>(base + l.masks);
+  S.counts = reinterpret_cast<int32_t *>(base + l.counts);
   S.info = reinterpret_cast<TileInfo *>(base + l.info);
   uint64_t *bars = reinterpret_cast<uint64_t *>(base + l.bars);
   S.full = bars;
@@ -210,10 +208,13 @@ __device__ __noinline__ void mma16s_role(const Fused16sArgs *ap, uint8_t *base, 
       tc_after();
       if (lane == 0) {
         const uint32_t a0 = su32(slot), b0 = su32(slot + S.slot_w);
+        // only the rows that have a segment s: the others' part of the tile is not written
+        const uint2 *m = S.masks + ((size_t)tb * a.list_chunks + s) * 4;
+        const uint4 off = make_uint4(~m[0].x, ~m[1].x, ~m[2].x, ~m[3].x);
         for (int ks = 0; ks < CHK / 16; ++ks) {
           const uint64_t ad = umma_desc(a0 + ks * 256, 128, sbo);
           const uint64_t bd = umma_desc(b0 + ks * 256, 128, sbo);
-          mma_h16(dacc, ad, bd, idesc0, (s > 0 || ks > 0) ? 1u : 0u);
+          mma_h16_rows(dacc, ad, bd, idesc0, off, (s > 0 || ks > 0) ? 1u : 0u);
         }
         mma_commit(su32(&S.empty[buf]));
       }
@@ -245,9 +246,7 @@ __device__ __noinline__ void epilogue16s_role(const Fused16sArgs *ap, uint8_t *b
   const QueryLaunch &q = a.q;
   const DevObject *objs = q.objs;
   const Smem16s S = carve16s<F, W>(a, base);
-  const int64_t n_tiles = (int64_t)q.s.meta[1];
   const int etid = tid - kEpiWarp0 * 32;
-  const int ew = etid >> 5;
   const int quarter = warp & 3;
   const int r = quarter * 32 + lane;
   const uint32_t w_sbo = (uint32_t)(W / 8) * 128u;  // SBO of a K = W core-matrix tile
@@ -257,203 +256,117 @@ __device__ __noinline__ void epilogue16s_role(const Fused16sArgs *ap, uint8_t *b
   uint32_t lw_phase = 0;
   bool lw_pending = false;
   int su_slot = -1;
+  TileFeed<false> feed(q, S.abort_flag, S.misc, 0, 0, etid);
 
-  auto fetch = [&]() -> int {
-    named_sync(2, kEpiThreads);
-    if (etid == 0) S.misc[0] = *S.abort_flag ? INT_MAX : atomicAdd(q.s.meta + 3, 1);
-    named_sync(2, kEpiThreads);
-    return S.misc[0];
-  };
-  auto slot_of_tile = [&](int tile) -> int { return q.s.tiles[3 * tile + 0]; };
-  auto setup = [&](int j, int tile) {
+  auto setup = [&](int j) {
     const int sb = j & 1;
-    if ((int64_t)tile >= n_tiles) {
+    if (feed.cnt < 0) {
       if (etid == 0) {
         S.info[sb].stop = 1;
         mbar_arrive(su32(&S.ready[sb]));
       }
       return;
     }
-    const int slot = q.s.tiles[3 * tile + 0];
-    const int start = q.s.tiles[3 * tile + 1];
-    const int cnt = q.s.tiles[3 * tile + 2];
-    const DevObject &ob = objs[slot];
-    if (slot != su_slot) {
+    if (feed.slot != su_slot) {
+      const DevObject &ob = objs[feed.slot];
       const float *src = reinterpret_cast<const float *>(ob.umma_h + ob.umma_bias_off);
       const int nb = ob.n_hidden * W + ob.n_out_pad;
       for (int k = etid; k < nb; k += kEpiThreads) S.bias[k] = __ldg(src + k);
       if (etid < LSNIF_MAX_LEVELS) S.res[etid] = (float)ob.res[etid];
-      su_slot = slot;
+      su_slot = feed.slot;
     }
-    if (etid == 0) S.misc[1] = 0;
-    named_sync(2, kEpiThreads);
-    int my_kk = 0;
-    uint32_t my_dm = 0u;
-    {
-      int ray = -1;
-      float t0v = 0.f, t1v = 0.f;
-      if (etid < cnt) {
-        ray = q.s.order[start + etid];
-        my_kk = q.s.k[ray];
-        my_dm = q.s.dup[ray];
-        const float2 tt = reinterpret_cast<const float2 *>(q.s.t01)[ray];
-        t0v = tt.x;
-        t1v = tt.y;
-      }
-      S.ray[sb * kTileM + etid] = ray;
-      S.t0[sb * kTileM + etid] = t0v;
-      S.t1[sb * kTileM + etid] = t1v;
-      const int wm = __reduce_max_sync(0xffffffffu, my_kk);
-      if (lane == 0) atomicMax(&S.misc[1], wm);
-    }
-    named_sync(2, kEpiThreads);
-    const int kmax = S.misc[1];
-    uint16_t *lst = S.list + (size_t)sb * a.list_chunks * kListStride;
-    uint32_t *ws = S.wsum + (size_t)sb * a.list_chunks * 4;
-    for (int s = 0; s < kmax; ++s) {
-      const uint32_t tot = __reduce_add_sync(0xffffffffu, row_counts(my_kk, my_dm, s));
-      if (lane == 0) ws[s * 4 + ew] = tot;
-    }
-    named_sync(2, kEpiThreads);
-    for (int s = 0; s < kmax; ++s) {
-      const uint32_t v = row_counts(my_kk, my_dm, s);
-      uint32_t incl = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const uint32_t y = __shfl_up_sync(0xffffffffu, incl, o);
-        if (lane >= o) incl += y;
-      }
-      uint32_t woff = 0, all = 0;
-#pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        const uint32_t x = ws[s * 4 + w];
-        all += x;
-        woff += w < ew ? x : 0u;
-      }
-      const uint32_t pos = incl - v + woff;
-      const int ngt = (int)(all & 1023u), nct = (int)((all >> 10) & 1023u);
-      uint16_t *Ls = lst + s * kListStride;
-      if (v & 1023u) {
-        const int pg = (int)(pos & 1023u);
-        if (v & (1023u << 10)) {  // entry point shared with the previous exit
-          Ls[pg] = (uint16_t)(etid | 128);
-          Ls[ngt + (int)((pos >> 10) & 1023u)] = (uint16_t)etid;
-        } else {
-          Ls[pg] = (uint16_t)etid;
-          Ls[pg + 1] = (uint16_t)(etid | 128);
-        }
-      } else {
-        const int pz = ngt + nct + (int)((pos >> 20) & 1023u);
-        Ls[pz] = (uint16_t)etid;
-        Ls[pz + 1] = (uint16_t)(etid | 128);
-      }
-    }
+    S.ray[sb * kTileM + etid] = feed.ray;
+    const int kmax = build_lists<true>(etid, feed.kk, feed.dm, S.list + (size_t)sb * a.list_chunks * kListStride,
+                                       S.masks + (size_t)sb * a.list_chunks * 4, S.counts + (size_t)sb * a.list_chunks,
+                                       S.misc, a.list_chunks);
     named_sync(2, kEpiThreads);
     if (etid == 0) {
       S.info[sb].kmax = kmax;
-      S.info[sb].slot = slot;
+      S.info[sb].slot = feed.slot;
       S.info[sb].stop = 0;
       mbar_arrive(su32(&S.ready[sb]));
     }
+    feed.stage = 0;
   };
 
-  int stop_at = INT_MAX;
-  {
-    const int t0i = fetch();
-    setup(0, t0i);
-    if ((int64_t)t0i >= n_tiles) stop_at = 0;
-  }
+  feed.finish();
+  int stop_at = feed.cnt < 0 ? 0 : INT_MAX;
+  setup(0);
   for (int i = 0; i < stop_at; ++i) {
     const int tb = i & 1;
     // set up tile i+1 now, unless it needs other biases: then after the
     // layers of tile i, which still read the current ones
-    const int tn = fetch();
-    const bool last = (int64_t)tn >= n_tiles;
-    const bool deferred = !last && slot_of_tile(tn) != su_slot;
-    if (!deferred) setup(i + 1, tn);
+    feed.finish();
+    const bool last = feed.cnt < 0, deferred = !last && feed.slot != su_slot;
+    if (!deferred) setup(i + 1);
     if (last) stop_at = i + 1;
 
     if (etid == 0) S.misc[2] = mbar_wait(su32(&S.accf[tb]), (uint32_t)((i >> 1) & 1), S.abort_flag) ? 0 : 1;
     named_sync(2, kEpiThreads);
     if (!S.misc[2]) {
       tc_after();
-      const TileInfo ti = S.info[tb];
-      const DevObject &ob = objs[ti.slot];
-      const int n_hidden = ob.n_hidden, n_out = ob.n_out, n_out_pad = ob.n_out_pad, n_mat = ob.n_mat,
-                act = ob.act;
+      const DevObject &ob = objs[S.info[tb].slot];
+      const int n_hidden = ob.n_hidden, n_out_pad = ob.n_out_pad;
+      const bool relu = ob.act == 0;
       const uint8_t *wsrc = ob.umma_h + (size_t)W * ob.n_in * 2;  // the later layers' FP16 weights
       const uint32_t dacc = tmem + (uint32_t)(tb * W);
       const uint32_t trow = dacc + ((uint32_t)(quarter * 32) << 16);
       const uint32_t act_col = tmem + (uint32_t)(2 * W);  // activation tile, lane 0
       const uint32_t tact = act_col + ((uint32_t)(quarter * 32) << 16);
-      for (int layer = 0; layer <= n_hidden; ++layer) {
-        const bool out_layer = layer == n_hidden;
+      const int ray = S.ray[tb * kTileM + r];
+      float tmin = 0.f, tmax = 0.f;
+      float2 t01 = make_float2(0.f, 0.f);
+      for (int layer = 0; layer < n_hidden; ++layer) {
         const float *bl = S.bias + layer * W;
-        if (!out_layer) {
-          const int N = (layer + 1 < n_hidden) ? W : n_out_pad;
-          const uint32_t wbytes = (uint32_t)N * W * 2u;
-          // the next layer's weights: the buffer's last reader (the previous
-          // layer's MMAs) has completed
-          if (etid == 0 && !lw_pending && !*S.abort_flag) {
-            bulk_copy(su32(S.lbuf), wsrc, wbytes, su32(S.lwfull));
-            lw_pending = true;
-            lw_phase = (uint32_t)(lw_ctr++ & 1);
-          }
-          wsrc += wbytes;
-#pragma unroll
-          for (int c0 = 0; c0 < W; c0 += 16) {
-            uint32_t v[16];
-            TMEM_LD16(trow + c0, (&v[0]));
-            tmem_wait_ld();
-            uint32_t hw[8];
-#pragma unroll
-            for (int u = 0; u < 8; ++u)
-              hw[u] = h2_sat(act_fn(__uint_as_float(v[2 * u]) + bl[c0 + 2 * u], act),
-                             act_fn(__uint_as_float(v[2 * u + 1]) + bl[c0 + 2 * u + 1], act));
-            TMEM_ST8(tact + (uint32_t)(c0 / 2), hw);
-          }
-          tmem_wait_st();
-          tc_before();
-          named_sync(2, kEpiThreads);
-          if (etid == 0) {
-            tc_after();
-            if (lw_pending && mbar_wait(su32(S.lwfull), lw_phase, S.abort_flag)) {
-              lw_pending = false;
-              const uint32_t b0 = su32(S.lbuf);
-              const uint32_t idesc = idesc_h16(N);
-              for (int ks = 0; ks < W / 16; ++ks)
-                mma_h16_ts(dacc, act_col + (uint32_t)(ks * 8), umma_desc(b0 + ks * 256, 128, w_sbo), idesc,
-                           ks > 0 ? 1u : 0u);
-              mma_commit(su32(S.layer));
-              mbar_wait(su32(S.layer), (uint32_t)(layer_ctr & 1), S.abort_flag);
-            }
-          }
-          ++layer_ctr;
-          named_sync(2, kEpiThreads);
-          tc_after();
-        } else {
-          // logits 16 columns at a time into a per-thread array, then decode
-          float z[64];
-#pragma unroll 1
-          for (int c0 = 0; c0 < n_out_pad; c0 += 16) {
-            uint32_t v[16];
-            TMEM_LD16(trow + c0, (&v[0]));
-            tmem_wait_ld();
-#pragma unroll
-            for (int u = 0; u < 16; ++u) z[c0 + u] = __uint_as_float(v[u]) + bl[c0 + u];
-          }
-          const int32_t ray = S.ray[tb * kTileM + r];
-          if (ray >= 0 && !*S.abort_flag)
-            decode_store(q.hits, ray, z, n_out, n_mat, S.t0[tb * kTileM + r], S.t1[tb * kTileM + r],
-                         q.rays.tmin[ray], q.rays.tmax[ray]);
+        const int N = (layer + 1 < n_hidden) ? W : n_out_pad;
+        const uint32_t wbytes = (uint32_t)N * W * 2u;
+        // the next layer's weights: the buffer's last reader (the previous
+        // layer's MMAs) has completed
+        if (etid == 0 && !lw_pending && !*S.abort_flag) {
+          bulk_copy(su32(S.lbuf), wsrc, wbytes, su32(S.lwfull));
+          lw_pending = true;
+          lw_phase = (uint32_t)(lw_ctr++ & 1);
         }
+        wsrc += wbytes;
+        if (relu) layer_activations<W, true, true>(trow, tact, tact, bl);
+        else layer_activations<W, true, false>(trow, tact, tact, bl);
+        tmem_wait_st();
+        tc_before();
+        named_sync(2, kEpiThreads);
+        bool issued = false;
+        if (etid == 0) {
+          tc_after();
+          if (lw_pending && mbar_wait(su32(S.lwfull), lw_phase, S.abort_flag)) {
+            lw_pending = false;
+            const uint32_t b0 = su32(S.lbuf);
+            const uint32_t idesc = idesc_h16(N);
+            for (int ks = 0; ks < W / 16; ++ks)
+              mma_h16_ts(dacc, act_col + (uint32_t)(ks * 8), umma_desc(b0 + ks * 256, 128, w_sbo), idesc,
+                         ks > 0 ? 1u : 0u);
+            mma_commit(su32(S.layer));
+            issued = true;
+          }
+        }
+        // while the MMAs run: the next tile but one, and the decode's inputs
+        if (!deferred && !last && feed.stage < 5) feed.step();
+        if (layer + 1 == n_hidden && ray >= 0) {
+          tmin = q.rays.tmin[ray];
+          tmax = q.rays.tmax[ray];
+          t01 = reinterpret_cast<const float2 *>(q.s.t01)[ray];
+        }
+        if (issued) mbar_wait(su32(S.layer), (uint32_t)(layer_ctr & 1), S.abort_flag);
+        ++layer_ctr;
+        named_sync(2, kEpiThreads);
+        tc_after();
       }
+      store_outputs<false>(q.hits, nullptr, trow, S.bias + n_hidden * W, ray, ray >= 0 && !*S.abort_flag, ob.n_out,
+                           n_out_pad, ob.n_mat, t01.x, t01.y, tmin, tmax);
     }
     tc_before();
     mbar_arrive(su32(&S.acce[tb]));
     if (deferred) {
       named_sync(2, kEpiThreads);  // every thread is done with the old biases
-      setup(i + 1, tn);
+      setup(i + 1);
     }
   }
   if (etid == 0) {
@@ -535,7 +448,8 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps16s) * 32, 1)
         cur_slot = ti.slot;
       }
       const uint16_t *s_lst = S.list + (size_t)tb * a.list_chunks * kListStride;
-      const uint32_t *s_ws = S.wsum + (size_t)tb * a.list_chunks * 4;
+      const uint2 *s_masks = S.masks + (size_t)tb * a.list_chunks * 4;
+      const int32_t *s_cnt = S.counts + (size_t)tb * a.list_chunks;
       const int G = (L * F) / 8;  // 16-byte column groups per point
       const int CHK = 2 * L * F;  // 16-bit columns per chunk
       const uint32_t a_sbo = (uint32_t)(CHK / 8) * 128u;
@@ -544,11 +458,11 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps16s) * 32, 1)
         const int c = chunk_ctr + s;
         const int buf = c % kNBuf16s, use = c / kNBuf16s;
         uint8_t *A = S.ring + buf * S.ring_stride;
-        uint32_t all = 0;
+        const int ngt = s_cnt[s];
+        int nct = 0;  // shared entry points, copied from the previous chunk
 #pragma unroll
-        for (int w = 0; w < 4; ++w) all += s_ws[s * 4 + w];
-        const int ngt = (int)(all & 1023u), nct = (int)((all >> 10) & 1023u);
-        const int n_gi = ngt * G, n_oi = (kListStride - ngt) * G;
+        for (int w = 0; w < 4; ++w) nct += __popc(s_masks[s * 4 + w].y);
+        const int n_gi = ngt * G, n_oi = nct * G;
         const int nb_g = (n_gi + 31) >> 5, nb_o = (n_oi + 31) >> 5;
         const int first_g = (warp - rot_g + NG) % NG, first_o = (warp - rot_o + NG) % NG;
         // the slot is free once the MMAs of chunk c - 2 are done and the
@@ -585,26 +499,20 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps16s) * 32, 1)
             *reinterpret_cast<uint4 *>(A + core_off(r, j * G + g, a_sbo)) = make_uint4(wv[0], wv[1], wv[2], wv[3]);
           }
         }
-        // copies (entry point = previous chunk's exit point) and zero fills
-        const int n_o = kListStride - ngt;
-        if (nct > 0 && first_o < nb_o) {  // copies read the previous chunk: it must be complete
+        // copies (entry point = previous chunk's exit point)
+        if (first_o < nb_o) {  // they read the previous chunk: it must be complete
           const int cq = c - 1;
           mbar_wait(su32(&S.full[cq % kNBuf16s]), (uint32_t)((cq / kNBuf16s) & 1), S.abort_flag);
         }
-        const float inv_o = 1.f / (float)max(n_o, 1);
+        const float inv_o = 1.f / (float)max(nct, 1);
         for (int b = first_o; b < nb_o; b += NG) {
           const int it = b * 32 + lane;
           if (it < n_oi) {
             const int g = __float2int_rz(((float)it + 0.5f) * inv_o);
-            const int t = it - g * n_o;
-            const int e = s_lst[s * kListStride + ngt + t];
-            const int r = e & 127, j = e >> 7;
-            uint4 outv = make_uint4(0u, 0u, 0u, 0u);
-            if (t < nct) {
-              const uint8_t *Ap = S.ring + ((c - 1) % kNBuf16s) * S.ring_stride;
-              outv = *reinterpret_cast<const uint4 *>(Ap + core_off(r, G + g, a_sbo));
-            }
-            *reinterpret_cast<uint4 *>(A + core_off(r, j * G + g, a_sbo)) = outv;
+            const int r = s_lst[s * kListStride + ngt + (it - g * nct)];
+            const uint8_t *Ap = S.ring + ((c - 1) % kNBuf16s) * S.ring_stride;
+            *reinterpret_cast<uint4 *>(A + core_off(r, g, a_sbo)) =
+                *reinterpret_cast<const uint4 *>(Ap + core_off(r, G + g, a_sbo));
           }
         }
         rot_g = (rot_g + nb_g) % NG;
@@ -660,7 +568,7 @@ static cudaError_t launch16s_shape(const Fused16sArgs &a, size_t smem, cudaStrea
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   // one persistent CTA per SM, but no more CTAs than the batch can have tiles
-  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, (int64_t)a.q.s.max_tiles));
+  const int grid = (int)std::max<int64_t>(1, std::min<int64_t>(sms, fused_items_max(a.q)));
   fused16s_kernel<F, W, NG, NL><<<grid, (NG + 1 + kEpiWarps16s) * 32, smem, st>>>(a);
   return cudaGetLastError();
 }

@@ -433,8 +433,10 @@ class Context:
         index per ray, -1 on a miss)."""
         import torch
         n = int(rays.shape[1])
-        res = self._alloc_hits(n, 0, False)
-        inst = torch.full((n,), -1, dtype=torch.int32, device=rays.device)
+        # the call writes every element
+        e = lambda *shape, dtype=torch.float32: torch.empty(shape, dtype=dtype, device=f"cuda:{self.device}")  # noqa: E731
+        res = QueryResult(e(n, dtype=torch.uint8), e(n), e(3, n), e(n, dtype=torch.int32), e(3, n), None)
+        inst = e(n, dtype=torch.int32)
         arr = self._instances(instances)
         rs = rays_struct(rays)
         hs = self.hits_struct(res)
