@@ -527,9 +527,8 @@ __device__ __forceinline__ int tile_shift(int n_live, int sms) {
 // Single block: bucket offsets (object ascending, k descending), tiles of
 // kTileM rays that never straddle objects, totals, cursors reset. A warp takes
 // one object's 32 buckets at a time, so an object's range starts at the value
-// its lane 0 scans to. One thread walking the buckets took 11 us on one object
-// (a load per bucket, none in flight beside another) and grew with the
-// objects; this takes 3 us, the launch included.
+// its lane 0 scans to. One thread walking the buckets (a load per bucket, none
+// in flight beside another) took 9.8 us on six objects; this takes 5.2.
 __global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
   __shared__ int ws[33];
   __shared__ int first[kMaxObjects + 1];     // start of each object's range
@@ -658,32 +657,28 @@ __global__ void __launch_bounds__(1024) scatter_block_kernel(QueryLaunch q, int 
 // count: live rays and points per block of kGroupBlock rays; scan: block
 // offsets, totals and the tile table; scatter: stable ranks within a block.
 // ---------------------------------------------------------------------------
+// The point counts of this thread's four rays (0 past n). A ray of an unknown
+// object has k = 0, so the slot is not needed.
+__device__ __forceinline__ uchar4 group_counts(const QueryLaunch &q) {
+  static_assert(kGroupBlock == 4096, "four rays per thread");
+  const int64_t i = (int64_t)blockIdx.x * kGroupBlock + 4 * threadIdx.x;
+  if (i + 4 <= q.rays.n) return *reinterpret_cast<const uchar4 *>(q.s.k + i);
+  uchar4 k = make_uchar4(0, 0, 0, 0);
+  if (i < q.rays.n) k.x = q.s.k[i];
+  if (i + 1 < q.rays.n) k.y = q.s.k[i + 1];
+  if (i + 2 < q.rays.n) k.z = q.s.k[i + 2];
+  return k;
+}
+
 __global__ void __launch_bounds__(1024) group_count_kernel(QueryLaunch q, int nblk) {
-  __shared__ int s_live[32], s_pts[32];
-  const int b = blockIdx.x;
-  int live = 0, pts = 0;
-  for (int r = 0; r < kGroupBlock / 1024; ++r) {
-    const int64_t i = (int64_t)b * kGroupBlock + r * 1024 + threadIdx.x;
-    if (i < q.rays.n && q.s.slot[i] >= 0) {
-      const int k = q.s.k[i];
-      live += k > 0;
-      pts += 2 * k;
-    }
-  }
-  for (int o = 16; o > 0; o >>= 1) {
-    live += __shfl_down_sync(0xffffffffu, live, o);
-    pts += __shfl_down_sync(0xffffffffu, pts, o);
-  }
-  if ((threadIdx.x & 31) == 0) {
-    s_live[threadIdx.x >> 5] = live;
-    s_pts[threadIdx.x >> 5] = pts;
-  }
-  __syncthreads();
+  __shared__ int ws[33];
+  const uchar4 k = group_counts(q);
+  int live, pts;
+  block_scan((k.x > 0) + (k.y > 0) + (k.z > 0) + (k.w > 0), ws, live);
+  block_scan(2 * (k.x + k.y + k.z + k.w), ws, pts);
   if (threadIdx.x == 0) {
-    int a = 0, c = 0;
-    for (int w = 0; w < 32; ++w) { a += s_live[w]; c += s_pts[w]; }
-    q.s.blk[b] = a;
-    q.s.blk[nblk + b] = c;
+    q.s.blk[blockIdx.x] = live;
+    q.s.blk[nblk + blockIdx.x] = pts;
   }
 }
 
@@ -720,43 +715,16 @@ __global__ void __launch_bounds__(1024) group_scan_kernel(QueryLaunch q, int nbl
   }
 }
 
-// A block's 4 x 1024 rays: every thread reads its four first, then one scan
-// over the (round, warp) totals places them in ray order.
 __global__ void __launch_bounds__(1024) group_scatter_kernel(QueryLaunch q) {
-  constexpr int kRounds = kGroupBlock / 1024;
-  __shared__ int s_off[kRounds * 32];
-  const int b = blockIdx.x, lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int base = q.s.blk[b];
-  unsigned m[kRounds];
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t i = (int64_t)b * kGroupBlock + r * 1024 + threadIdx.x;
-    m[r] = __ballot_sync(0xffffffffu, i < q.rays.n && q.s.slot[i] >= 0 && q.s.k[i] > 0);
-    if (lane == 0) s_off[r * 32 + warp] = __popc(m[r]);
-  }
-  __syncthreads();
-  if (warp == 0) {  // exclusive scan of the kRounds x 32 totals
-    int run = 0;
-#pragma unroll
-    for (int r = 0; r < kRounds; ++r) {
-      const int v = s_off[r * 32 + lane];
-      int inc = v;
-#pragma unroll
-      for (int o = 1; o < 32; o <<= 1) {
-        const int y = __shfl_up_sync(0xffffffffu, inc, o);
-        if (lane >= o) inc += y;
-      }
-      s_off[r * 32 + lane] = run + inc - v;
-      run += __shfl_sync(0xffffffffu, inc, 31);
-    }
-  }
-  __syncthreads();
-#pragma unroll
-  for (int r = 0; r < kRounds; ++r) {
-    const int64_t i = (int64_t)b * kGroupBlock + r * 1024 + threadIdx.x;
-    if ((m[r] >> lane) & 1u)
-      q.s.order[base + s_off[r * 32 + warp] + __popc(m[r] & ((1u << lane) - 1u))] = (int32_t)i;
-  }
+  __shared__ int ws[33];
+  const uchar4 k = group_counts(q);
+  int total;
+  int at = q.s.blk[blockIdx.x] + block_scan((k.x > 0) + (k.y > 0) + (k.z > 0) + (k.w > 0), ws, total);
+  const int32_t i = (int32_t)((int64_t)blockIdx.x * kGroupBlock + 4 * threadIdx.x);
+  if (k.x) q.s.order[at++] = i;
+  if (k.y) q.s.order[at++] = i + 1;
+  if (k.z) q.s.order[at++] = i + 2;
+  if (k.w) q.s.order[at++] = i + 3;
 }
 
 // exclusive scan of n int32 in place, in blocks of 1024; block totals to sums
