@@ -230,8 +230,10 @@ struct TrainBuffers {
   float *pre;       // B x width x n_hidden (pre-activation)
   float *Z;         // B x n_out
   float *dZ;        // B x n_out
-  float *dA;        // B x max(width, n_in) scratch
-  float *dB;        // B x max(width, n_in) scratch
+  float *dA, *dB;   // B x width scratch
+  // scratch of the fused input gradient and scatter, NULL where it is not used
+  void *w0t;
+  float *dense;
   float *pts;       // B x H x 3
   float *t01;       // B x 2
   int32_t *k;       // B
@@ -248,6 +250,21 @@ struct TrainBuffers {
   float *grad_tab;  // L x T x F
   float *m_mlp, *v_mlp, *m_tab, *v_tab;
 };
+
+// Scratch of the fused input gradient and scatter (train_scatter.cu); ok: the
+// shape is covered
+struct InputScatterPlan {
+  bool ok;
+  size_t w0t_bytes, dense_bytes;
+  int n_dense;
+  int64_t dense_stride;
+  int32_t dense_off[LSNIF_MAX_LEVELS];
+};
+InputScatterPlan input_scatter_plan(const DevObject &h);
+// dX = dY . W0 (tensor cores, two-term BF16) scattered into the table gradients
+cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int64_t B, const float *dY, const float *W0,
+                                 const int32_t *k, const float *pts, float *gtab, void *w0t, float *dense, int *err,
+                                 cudaStream_t st);
 
 cudaError_t launch_make_training_rays(const DevObject *dobj, const DevObject &h, const float *u, int64_t n,
                                       int64_t n_outside, float *rays_out, uint8_t *surface,

@@ -584,31 +584,47 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
       fi = fo;
     }
   }
-  const int ks = (int)std::min<int64_t>(256, std::max<int64_t>(1, B / 1024));
+  // Ranges the batch is split into for the weight gradients: 1024 rays each,
+  // shorter ones where a small batch would leave SMs idle (two CTAs per SM over
+  // the product's column tiles, at least 128 rays each). 16,384 rays on the
+  // 144-128x2-12 network: the three products 174 us in ranges of 1024, 50 us so.
+  auto ranges = [&](int n) {
+    const int64_t tiles = (n + 63) / 64;
+    return (int)std::min<int64_t>(
+        256, std::max<int64_t>({1, B / 1024, std::min<int64_t>((304 + tiles - 1) / tiles, B / 128)}));
+  };
   const float *d = tb.dZ;  // gradient w.r.t. the current layer's output (pre-activation)
   int dcols = NO;
   for (int l = NH; l >= 0; --l) {
     const int fi = l == 0 ? NI : W;
     const float *hin = l == 0 ? tb.feats : tb.acts + (size_t)(l - 1) * B * W;
     // dW = d^T . hin  (dcols x fi), split over the batch
-    mm(dcols, fi, (int)B, d, dcols, 1, hin, fi, 0, gW[l], fi, 1, nullptr, nullptr, nullptr, 0, ks);
+    mm(dcols, fi, (int)B, d, dcols, 1, hin, fi, 0, gW[l], fi, 1, nullptr, nullptr, nullptr, 0, ranges(fi));
     {
       const int threads = dcols * std::max(1, 256 / dcols);
-      colsum_kernel<<<152 * 8, threads, threads * sizeof(float), st>>>(d, B, dcols, gb[l]);
+      // 16 rows or more per thread: every block ends with an atomic per column
+      const int per = threads / dcols;
+      colsum_kernel<<<grid_for(B / 16, per, 152 * 8), threads, threads * sizeof(float), st>>>(d, B, dcols, gb[l]);
     }
     // gradient w.r.t. the layer input: d . W_l (B x fi); for hidden inputs
     // multiply by act'(pre of layer l-1)
     float *dn = (l % 2 == 0) ? tb.dA : tb.dB;
-    if (l > 0)
+    if (l > 0) {
       mm((int)B, fi, dcols, d, dcols, 0, Wl[l], fi, 0, dn, fi, 4, nullptr, nullptr, tb.pre + (size_t)(l - 1) * B * W,
          h.act);
-    else
-      mm((int)B, fi, dcols, d, dcols, 0, Wl[l], fi, 0, dn, fi, 0);
+    } else if (tc && tb.w0t) {
+      e = launch_input_scatter(dobj, h, B, d, Wl[0], tb.k, tb.pts, tb.grad_tab, tb.w0t, tb.dense, err, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      // dX takes the place of the features, which are not needed any more;
+      // then its scatter into the table gradients
+      mm((int)B, fi, dcols, d, dcols, 0, Wl[l], fi, 0, tb.feats, fi, 0);
+      train_scatter_kernel<<<grid_for(B * h.H * h.L, 256, 152 * 32), 256, 0, st>>>(dobj, B, tb.k, tb.pts, tb.feats,
+                                                                                   tb.grad_tab);
+    }
     d = dn;
     dcols = fi;
   }
-  // d is dX (B x n_in): scatter into the table gradients
-  train_scatter_kernel<<<grid_for(B * h.H * h.L, 256, 152 * 32), 256, 0, st>>>(dobj, B, tb.k, tb.pts, d, tb.grad_tab);
   if (opts.apply_update) {
     const double c1 = 1.0 - std::pow((double)opts.beta1, (double)step);
     const double c2 = 1.0 - std::pow((double)opts.beta2, (double)step);

@@ -64,8 +64,18 @@ static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
   TALLOC(pre, float *, 4 * (size_t)B * W * c.n_hidden);
   TALLOC(Z, float *, 4 * (size_t)B * NO);
   TALLOC(dZ, float *, 4 * (size_t)B * NO);
-  TALLOC(dA, float *, 4 * (size_t)B * std::max(W, NI));
-  TALLOC(dB, float *, 4 * (size_t)B * std::max(W, NI));
+  TALLOC(dA, float *, 4 * (size_t)B * W);
+  TALLOC(dB, float *, 4 * (size_t)B * W);
+  // The fused input gradient and scatter takes its scratch out of what the
+  // two buffers above held for dX (n_in columns each) before it: a batch
+  // whose dX is smaller than the scratch keeps the separate kernels.
+  const InputScatterPlan plan = input_scatter_plan(o->d);
+  tb.w0t = nullptr;
+  tb.dense = nullptr;
+  if (plan.ok && NI > W && plan.w0t_bytes + plan.dense_bytes + 1024 <= 8 * (size_t)B * (NI - W)) {
+    TALLOC(w0t, void *, plan.w0t_bytes);
+    TALLOC(dense, float *, std::max<size_t>(plan.dense_bytes, 16));
+  }
   TALLOC(pts, float *, 12 * (size_t)B * c.H);
   TALLOC(t01, float *, 8 * (size_t)B);
   TALLOC(k, int32_t *, 4 * (size_t)B);
