@@ -227,7 +227,7 @@ cudaError_t launch_mlp_fused(const DevObject *dobj, const DevObject &host_obj, c
 struct TrainBuffers {
   float *feats;     // B x n_in (FP32)
   float *acts;      // B x width x n_hidden (post-activation)
-  float *pre;       // B x width x n_hidden (pre-activation)
+  float *pre;       // B x width x n_hidden: pre-activations, or the gradients of them (train_chain.cu)
   float *Z;         // B x n_out
   float *dZ;        // B x n_out
   float *dA, *dB;   // B x width scratch
@@ -250,6 +250,14 @@ struct TrainBuffers {
   float *grad_tab;  // L x T x F
   float *m_mlp, *v_mlp, *m_tab, *v_tab;
 };
+
+// Layers after the first, loss and the backward pass down to the first layer's
+// pre-activations in one kernel (train_chain.cu): acts[0] given, acts[1..],
+// grads[0..] (n_hidden x B x width each) and dZ written, loss[0..5] summed
+bool train_chain_supported(const DevObject &h);
+cudaError_t launch_train_chain(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k, float *acts,
+                               float *grads, float *dZ, const lsnif_labels &lab, float *loss, int *err,
+                               cudaStream_t st);
 
 // Scratch of the fused input gradient and scatter (train_scatter.cu); ok: the
 // shape is covered
@@ -279,7 +287,7 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
 // C[M x N] = op(A) . op(B) on the tensor cores (two-term BF16, FP32
 // accumulation), op(A)[m][k] = tA ? A[k lda + m] : A[m lda + k], op(B)[k][n] =
 // tB ? B[n ldb + k] : B[k ldb + n]; mode 0 store, 1 atomic add (k_split > 1
-// allowed), 2 + bias[n] -> C, act -> post, 3 + bias[n], 4 times act'(aux) (train_gemm.cu)
+// allowed), 2 + bias[n] -> C, act -> post, 3 + bias[n], 4 times act'(aux), 5 act of + bias[n] (train_gemm.cu)
 cudaError_t launch_tc_gemm(cudaStream_t st, int M, int N, int K, const float *A, int lda, int tA, const float *B,
                            int ldb, int tB, float *C, int ldc, int mode, const float *bias, float *post,
                            const float *aux, int act, int k_split, int *err);

@@ -561,16 +561,25 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
     p += (size_t)fo * fan_in + fo;
     fan_in = fo;
   }
-  const float *in = tb.feats;
-  int K = NI;
-  for (int l = 0; l < NH; ++l) {
-    float *pre = tb.pre + (size_t)l * B * W, *post = tb.acts + (size_t)l * B * W;
-    mm((int)B, W, K, in, K, 0, Wl[l], K, 1, pre, W, 2, bl[l], post, nullptr, h.act);
-    in = post;
-    K = W;
+  // The layers after the first, the loss and their backward pass in one
+  // kernel where the shape allows; else a product per layer and direction.
+  const bool chain = tc && train_chain_supported(h);
+  if (chain) {
+    mm((int)B, W, NI, tb.feats, NI, 0, Wl[0], NI, 1, tb.acts, W, 5, bl[0], nullptr, nullptr, h.act);
+    e = launch_train_chain(dobj, h, B, tb.k, tb.acts, tb.pre, tb.dZ, lab, tb.loss, err, st);
+    if (e != cudaSuccess) return e;
+  } else {
+    const float *in = tb.feats;
+    int K = NI;
+    for (int l = 0; l < NH; ++l) {
+      float *pre = tb.pre + (size_t)l * B * W, *post = tb.acts + (size_t)l * B * W;
+      mm((int)B, W, K, in, K, 0, Wl[l], K, 1, pre, W, 2, bl[l], post, nullptr, h.act);
+      in = post;
+      K = W;
+    }
+    mm((int)B, NO, W, in, W, 0, Wl[NH], W, 1, tb.Z, NO, 3, bl[NH]);
+    loss_kernel<<<grid_for(B, 256, 152 * 8), 256, 0, st>>>(dobj, B, tb.k, tb.Z, lab, tb.dZ, tb.loss, tb.loss + 6);
   }
-  mm((int)B, NO, W, in, W, 0, Wl[NH], W, 1, tb.Z, NO, 3, bl[NH]);
-  loss_kernel<<<grid_for(B, 256, 152 * 8), 256, 0, st>>>(dobj, B, tb.k, tb.Z, lab, tb.dZ, tb.loss, tb.loss + 6);
   // backward through the network; gradient layout mirrors the packed weights
   float *gW[LSNIF_MAX_HIDDEN + 1], *gb[LSNIF_MAX_HIDDEN + 1];
   {
@@ -609,7 +618,9 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
     // gradient w.r.t. the layer input: d . W_l (B x fi); for hidden inputs
     // multiply by act'(pre of layer l-1)
     float *dn = (l % 2 == 0) ? tb.dA : tb.dB;
-    if (l > 0) {
+    if (chain && l > 0) {
+      dn = tb.pre + (size_t)(l - 1) * B * W;
+    } else if (l > 0) {
       mm((int)B, fi, dcols, d, dcols, 0, Wl[l], fi, 0, dn, fi, 4, nullptr, nullptr, tb.pre + (size_t)(l - 1) * B * W,
          h.act);
     } else if (tc && tb.w0t) {

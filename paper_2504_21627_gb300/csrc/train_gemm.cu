@@ -324,6 +324,7 @@ __global__ void __launch_bounds__(kGThreads) tc_gemm_kernel(const __grid_constan
       else if (g.mode == 1) { if (nchunks > 0) atomicAdd(g.C + o, x); }
       else if (g.mode == 2) { x += g.bias[gn]; g.C[o] = x; g.post[o] = act_fn(x, g.act); }
       else if (g.mode == 3) g.C[o] = x + g.bias[gn];
+      else if (g.mode == 5) g.C[o] = act_fn(x + g.bias[gn], g.act);
       else g.C[o] = x * act_grad(g.aux[o], g.act);
     }
     __syncthreads();
