@@ -213,13 +213,18 @@ __global__ void label_kernel(const DevObject *dobj, RaysArg r, lsnif_labels L) {
 // no occupied voxel stay zero.
 // ---------------------------------------------------------------------------
 template <int F>
-__device__ __forceinline__ void feature_level(const DevObject &ob, int l, const float3 &p, float *xo) {
+__device__ __forceinline__ void feature_level(const DevObject &ob, int l, const float3 &p, float *xo, bool both) {
   const float *tl = ob.tab32 + (size_t)l * (ob.mask + 1) * F;
   float f[F];
-  if constexpr (F == 2) encode_level_f32_if<F>(tl, ob.mask, p, (float)ob.res[l], true, f);
-  else encode_level<float, F>(tl, ob.mask, p, (float)ob.res[l], f);
+  if constexpr (F == 1) encode_level<float, F>(tl, ob.mask, p, (float)ob.res[l], f);
+  else encode_level_f32_if<F>(tl, ob.mask, p, (float)ob.res[l], true, f);
+  float *const next = xo + ob.L * F;  // the next point's features
 #pragma unroll
   for (int j = 0; j < F; ++j) xo[j] = f[j];
+  if (both) {
+#pragma unroll
+    for (int j = 0; j < F; ++j) next[j] = f[j];
+  }
 }
 
 // (ray i, point h, level l) of work item e = (i H + h) L + l, with 32-bit
@@ -250,15 +255,20 @@ __global__ void train_features_kernel(const DevObject *dobj, int64_t B, const in
     int h, l;
     split_item(e, narrow, H, L, i, h, l);
     float *xo = X + i * ob.n_in + ((size_t)h * L + l) * F;
-    if (h >= 2 * k[i]) {
+    const int n_pts = 2 * k[i];
+    if (h >= n_pts) {
       for (int j = 0; j < F; ++j) xo[j] = 0.f;
       continue;
     }
     const float *pp = pts + (i * H + h) * 3;
     const float3 p = make_float3(pp[0], pp[1], pp[2]);
-    if (F == 2) feature_level<2>(ob, l, p, xo);
-    else if (F == 4) feature_level<4>(ob, l, p, xo);
-    else feature_level<1>(ob, l, p, xo);
+    // an entry point (even h > 0) equal to the exit point before it has that
+    // point's features, which its thread writes to both places
+    if (h > 0 && (h & 1) == 0 && pp[-3] == p.x && pp[-2] == p.y && pp[-1] == p.z) continue;
+    const bool both = (h & 1) == 1 && h + 1 < n_pts && pp[3] == p.x && pp[4] == p.y && pp[5] == p.z;
+    if (F == 2) feature_level<2>(ob, l, p, xo, both);
+    else if (F == 4) feature_level<4>(ob, l, p, xo, both);
+    else feature_level<1>(ob, l, p, xo, both);
   }
 }
 
