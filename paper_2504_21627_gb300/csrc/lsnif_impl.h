@@ -225,18 +225,19 @@ cudaError_t launch_mlp_fused(const DevObject *dobj, const DevObject &host_obj, c
 
 // ---- training (train.cu) ----
 struct TrainBuffers {
-  float *feats;     // B x n_in (FP32)
+  float *feats;     // B x n_in: FP32, or two-term BF16 tiles (train_layer0.cu)
   float *acts;      // B x width x n_hidden (post-activation)
   float *pre;       // B x width x n_hidden: pre-activations, or the gradients of them (train_chain.cu)
   float *Z;         // B x n_out
   float *dZ;        // B x n_out
   float *dA, *dB;   // B x width scratch
-  // scratch of the fused input gradient and scatter, NULL where it is not used
+  // scratch of the first layer's own kernels, NULL where they are not used
   void *w0t;
   float *dense;
+  int32_t *order;   // B: ray of a row, and kBuckets counters
   float *pts;       // B x H x 3
   float *t01;       // B x 2
-  int32_t *k;       // B
+  int32_t *k;       // B: segments of a row's ray
   // the query traversal's own outputs for the batch: one-byte point counts
   // (widened into k), shared-point bits, object slots, its histogram
   // (kMaxSlots x kBuckets) and counters
@@ -255,9 +256,9 @@ struct TrainBuffers {
 // pre-activations in one kernel (train_chain.cu): acts[0] given, acts[1..],
 // grads[0..] (n_hidden x B x width each) and dZ written, loss[0..5] summed
 bool train_chain_supported(const DevObject &h);
-cudaError_t launch_train_chain(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k, float *acts,
-                               float *grads, float *dZ, const lsnif_labels &lab, float *loss, int *err,
-                               cudaStream_t st);
+cudaError_t launch_train_chain(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k,
+                               const int32_t *order, float *acts, float *grads, float *dZ, const lsnif_labels &lab,
+                               float *loss, int *err, cudaStream_t st);
 
 // Scratch of the fused input gradient and scatter (train_scatter.cu); ok: the
 // shape is covered
@@ -269,10 +270,24 @@ struct InputScatterPlan {
   int32_t dense_off[LSNIF_MAX_LEVELS];
 };
 InputScatterPlan input_scatter_plan(const DevObject &h);
+// the first layer's weights (W x n_in FP32) as two-term BF16, transposed, per segment
+cudaError_t launch_build_w0t(const DevObject &h, const float *W0, void *w0t, cudaStream_t st);
 // dX = dY . W0 (tensor cores, two-term BF16) scattered into the table gradients
-cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int64_t B, const float *dY, const float *W0,
-                                 const int32_t *k, const float *pts, float *gtab, void *w0t, float *dense, int *err,
-                                 cudaStream_t st);
+cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int64_t B, const float *dY,
+                                 const void *w0t, const int32_t *k, const int32_t *order, const float *pts,
+                                 float *gtab, float *dense, int *err, cudaStream_t st);
+
+// The first layer over rays in order of their segment count (train_layer0.cu):
+// row -> ray and segment count; features as tiles of two-term BF16 operands
+// (whole tiles of kTileM rows); forward product; weight and bias gradients
+cudaError_t launch_order_rays(const uint8_t *k8, int64_t B, const int32_t *hist, int32_t *cursor, int32_t *k,
+                              int32_t *order, float *live, cudaStream_t st);
+cudaError_t launch_tile_features(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k,
+                                 const int32_t *order, const float *pts, void *x, cudaStream_t st);
+cudaError_t launch_layer0(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k, const void *x,
+                          const void *w0t, const float *bias, float *acts, int *err, cudaStream_t st);
+cudaError_t launch_layer0_grad(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k, const void *x,
+                               const float *dY, float *gW, float *gb, int *err, cudaStream_t st);
 
 cudaError_t launch_make_training_rays(const DevObject *dobj, const DevObject &h, const float *u, int64_t n,
                                       int64_t n_outside, float *rays_out, uint8_t *surface,

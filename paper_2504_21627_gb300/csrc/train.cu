@@ -558,8 +558,22 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
   int launches = 0;
   cudaError_t e = launch_trace(q, &launches);
   if (e != cudaSuccess) return e;
-  widen_count_kernel<<<grid_for(B, 256, 152 * 4), 256, 0, st>>>(tb.k8, B, tb.k, tb.loss + 6);
-  train_features_kernel<<<grid_for(B * h.H * h.L, 256, 152 * 32), 256, 0, st>>>(dobj, B, tb.k, tb.pts, tb.feats);
+  // The layers after the first, the loss and their backward pass in one
+  // kernel where the shape allows, else a product per layer and direction; the
+  // first layer's own kernels, over rays ordered by segment count, where their
+  // scratch is there too.
+  const bool chain = tc && train_chain_supported(h);
+  const bool own = chain && tb.w0t;
+  const int32_t *order = own ? tb.order : nullptr;  // ray of a row
+  if (own) {
+    e = launch_order_rays(tb.k8, B, tb.counts + (size_t)(n_slots - 1) * kBuckets, tb.order + B, tb.k, tb.order,
+                          tb.loss + 6, st);
+    if (e == cudaSuccess) e = launch_tile_features(dobj, h, B, tb.k, order, tb.pts, tb.feats, st);
+    if (e != cudaSuccess) return e;
+  } else {
+    widen_count_kernel<<<grid_for(B, 256, 152 * 4), 256, 0, st>>>(tb.k8, B, tb.k, tb.loss + 6);
+    train_features_kernel<<<grid_for(B * h.H * h.L, 256, 152 * 32), 256, 0, st>>>(dobj, B, tb.k, tb.pts, tb.feats);
+  }
   // forward: pre[l], acts[l] (B x W each), logits Z
   const float *p = h.mlp32;
   const float *Wl[LSNIF_MAX_HIDDEN + 1], *bl[LSNIF_MAX_HIDDEN + 1];
@@ -571,12 +585,18 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
     p += (size_t)fo * fan_in + fo;
     fan_in = fo;
   }
-  // The layers after the first, the loss and their backward pass in one
-  // kernel where the shape allows; else a product per layer and direction.
-  const bool chain = tc && train_chain_supported(h);
+  if (tc && tb.w0t) {
+    e = launch_build_w0t(h, Wl[0], tb.w0t, st);
+    if (e != cudaSuccess) return e;
+  }
   if (chain) {
-    mm((int)B, W, NI, tb.feats, NI, 0, Wl[0], NI, 1, tb.acts, W, 5, bl[0], nullptr, nullptr, h.act);
-    e = launch_train_chain(dobj, h, B, tb.k, tb.acts, tb.pre, tb.dZ, lab, tb.loss, err, st);
+    if (own) {
+      e = launch_layer0(dobj, h, B, tb.k, tb.feats, tb.w0t, bl[0], tb.acts, err, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      mm((int)B, W, NI, tb.feats, NI, 0, Wl[0], NI, 1, tb.acts, W, 5, bl[0], nullptr, nullptr, h.act);
+    }
+    e = launch_train_chain(dobj, h, B, tb.k, order, tb.acts, tb.pre, tb.dZ, lab, tb.loss, err, st);
     if (e != cudaSuccess) return e;
   } else {
     const float *in = tb.feats;
@@ -617,9 +637,12 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
   for (int l = NH; l >= 0; --l) {
     const int fi = l == 0 ? NI : W;
     const float *hin = l == 0 ? tb.feats : tb.acts + (size_t)(l - 1) * B * W;
-    // dW = d^T . hin  (dcols x fi), split over the batch
-    mm(dcols, fi, (int)B, d, dcols, 1, hin, fi, 0, gW[l], fi, 1, nullptr, nullptr, nullptr, 0, ranges(fi));
-    {
+    // dW = d^T . hin  (dcols x fi), split over the batch, and db
+    if (l == 0 && own) {
+      e = launch_layer0_grad(dobj, h, B, tb.k, tb.feats, d, gW[0], gb[0], err, st);
+      if (e != cudaSuccess) return e;
+    } else {
+      mm(dcols, fi, (int)B, d, dcols, 1, hin, fi, 0, gW[l], fi, 1, nullptr, nullptr, nullptr, 0, ranges(fi));
       const int threads = dcols * std::max(1, 256 / dcols);
       // 16 rows or more per thread: every block ends with an atomic per column
       const int per = threads / dcols;
@@ -634,7 +657,7 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
       mm((int)B, fi, dcols, d, dcols, 0, Wl[l], fi, 0, dn, fi, 4, nullptr, nullptr, tb.pre + (size_t)(l - 1) * B * W,
          h.act);
     } else if (tc && tb.w0t) {
-      e = launch_input_scatter(dobj, h, B, d, Wl[0], tb.k, tb.pts, tb.grad_tab, tb.w0t, tb.dense, err, st);
+      e = launch_input_scatter(dobj, h, B, d, tb.w0t, tb.k, order, tb.pts, tb.grad_tab, tb.dense, err, st);
       if (e != cudaSuccess) return e;
     } else {
       // dX takes the place of the features, which are not needed any more;

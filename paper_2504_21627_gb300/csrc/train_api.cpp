@@ -59,20 +59,27 @@ static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
 #define TALLOC(field, type, bytes)                                                   \
   if ((rc = train_alloc(ctx, o, (bytes), &p, "training buffers")) != LSNIF_OK) return rc; \
   tb.field = (type)p;
-  TALLOC(feats, float *, 4 * (size_t)B * NI);
+  // The first layer's own kernels (train_layer0.cu, train_scatter.cu) take
+  // their scratch out of what the buffers dA and dB held for dX (n_in columns
+  // each) before them: a batch whose dX is smaller than the scratch keeps the
+  // separate kernels.
+  const InputScatterPlan plan = input_scatter_plan(o->d);
+  const size_t rows = ((size_t)B + kTileM - 1) / kTileM * kTileM, order_bytes = 4 * ((size_t)B + kBuckets);
+  const bool own = plan.ok && NI > W &&
+                   plan.w0t_bytes + plan.dense_bytes + order_bytes + 4 * (rows - B) * NI + 1024 <=
+                       8 * (size_t)B * (NI - W);
+  TALLOC(feats, float *, 4 * (own ? rows : (size_t)B) * NI);
   TALLOC(acts, float *, 4 * (size_t)B * W * c.n_hidden);
   TALLOC(pre, float *, 4 * (size_t)B * W * c.n_hidden);
   TALLOC(Z, float *, 4 * (size_t)B * NO);
   TALLOC(dZ, float *, 4 * (size_t)B * NO);
   TALLOC(dA, float *, 4 * (size_t)B * W);
   TALLOC(dB, float *, 4 * (size_t)B * W);
-  // The fused input gradient and scatter takes its scratch out of what the
-  // two buffers above held for dX (n_in columns each) before it: a batch
-  // whose dX is smaller than the scratch keeps the separate kernels.
-  const InputScatterPlan plan = input_scatter_plan(o->d);
   tb.w0t = nullptr;
   tb.dense = nullptr;
-  if (plan.ok && NI > W && plan.w0t_bytes + plan.dense_bytes + 1024 <= 8 * (size_t)B * (NI - W)) {
+  tb.order = nullptr;
+  if (own) {
+    TALLOC(order, int32_t *, order_bytes);
     TALLOC(w0t, void *, plan.w0t_bytes);
     TALLOC(dense, float *, std::max<size_t>(plan.dense_bytes, 16));
   }

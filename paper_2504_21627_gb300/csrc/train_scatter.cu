@@ -5,7 +5,7 @@
 //
 // Before, a product wrote dX (B x n_in FP32, 604 MB on the torus batch of
 // 2^18) and a kernel with a thread per (ray, point, level) read it back: 454 +
-// 1244 us, against 952 us here. What bounds this form: L2's reductions (68% of
+// 1244 us, against 952 us here, 805 us over rays in order of their segment count. What bounds this form: L2's reductions (68% of
 // their sector rate). So
 //   - the two x corners of a cell go as one 16-byte reduction where they lie in
 //     one aligned pair (every even cell; F = 2): six reductions per point and
@@ -51,6 +51,7 @@ struct ScatterArgs {
   const float *dY;       // B x W
   const uint8_t *w0t;    // per segment: hi tile, lo tile (CHK x W BF16 each, K-major core matrices)
   const int32_t *k;
+  const int32_t *order;  // ray of a row (NULL: the row itself)
   const float *pts;
   float *gtab;
   float *dense;          // kReplicas copies of the dense levels' lattices
@@ -160,16 +161,13 @@ __global__ void __launch_bounds__(kSThreads, HC <= 16 ? 3 : 1) input_scatter_ker
     const int m = __reduce_max_sync(0xffffffffu, kk);
     if (lane == 0 && half == 0) atomicMax(&s_kmax, m);
   }
-  // dY -> two-term BF16; an item is one row's 8 columns (two 16-byte loads),
+  // dY -> two-term BF16; an item is one row's 8 columns,
   // and a quarter-warp stores one whole core matrix
   for (int it = tid; it < kTileM * KG; it += kSThreads) {
     const int r = (it & 7) + (it / (8 * KG)) * 8, g = (it >> 3) % KG;
     float v[8] = {0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f, 0.f};
     if (r < rows) {
-      const float4 *src = reinterpret_cast<const float4 *>(a.dY + (r0 + r) * W + g * 8);
-      const float4 x = __ldg(src), y = __ldg(src + 1);
-      v[0] = x.x; v[1] = x.y; v[2] = x.z; v[3] = x.w;
-      v[4] = y.x; v[5] = y.y; v[6] = y.z; v[7] = y.w;
+      load8(a.dY + (r0 + r) * W + g * 8, v);
     }
     uint32_t hw[4], lw[4];
 #pragma unroll
@@ -217,7 +215,8 @@ __global__ void __launch_bounds__(kSThreads, HC <= 16 ? 3 : 1) input_scatter_ker
     if (!s_abort) issued = 1;
   }
   float *gdense = a.dense + (size_t)(blockIdx.x % kReplicas) * a.dense_stride;
-  const float *P = a.pts + (r0 + min(row, rows - 1)) * ob.H * 3;
+  const int64_t r = r0 + min(row, rows - 1);
+  const float *P = a.pts + (a.order ? a.order[r] : r) * ob.H * 3;
   const uint32_t trow = tmem + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(half * HC);
   constexpr int LH = HC / F;  // levels of a warp
   for (int s = 0; s <= kmax && kmax > 0; ++s) {
@@ -357,9 +356,14 @@ InputScatterPlan input_scatter_plan(const DevObject &h) {
   return p;
 }
 
-cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int64_t B, const float *dY, const float *W0,
-                                 const int32_t *k, const float *pts, float *gtab, void *w0t, float *dense, int *err,
-                                 cudaStream_t st) {
+cudaError_t launch_build_w0t(const DevObject &h, const float *W0, void *w0t, cudaStream_t st) {
+  build_w0t_kernel<<<152, 256, 0, st>>>(W0, h.width, h.n_in, 2 * h.L * h.F, static_cast<uint8_t *>(w0t));
+  return cudaGetLastError();
+}
+
+cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int64_t B, const float *dY,
+                                 const void *w0t, const int32_t *k, const int32_t *order, const float *pts,
+                                 float *gtab, float *dense, int *err, cudaStream_t st) {
   const InputScatterPlan p = input_scatter_plan(h);
   ScatterArgs a{};
   a.obj = dobj;
@@ -369,6 +373,7 @@ cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int6
   a.dY = dY;
   a.w0t = static_cast<const uint8_t *>(w0t);
   a.k = k;
+  a.order = order;
   a.pts = pts;
   a.gtab = gtab;
   a.dense = dense;
@@ -378,7 +383,6 @@ cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int6
   a.err = err;
   cudaError_t e = p.dense_bytes ? cudaMemsetAsync(dense, 0, p.dense_bytes, st) : cudaSuccess;
   if (e != cudaSuccess) return e;
-  build_w0t_kernel<<<152, 256, 0, st>>>(W0, h.width, h.n_in, 2 * a.LF, static_cast<uint8_t *>(w0t));
   if (h.F == 2) e = a.LF == 16 ? launch_shape<2, 8>(a, st) : a.LF == 32 ? launch_shape<2, 16>(a, st) : launch_shape<2, 32>(a, st);
   else e = a.LF == 16 ? launch_shape<4, 8>(a, st) : a.LF == 32 ? launch_shape<4, 16>(a, st) : launch_shape<4, 32>(a, st);
   if (e != cudaSuccess) return e;

@@ -77,3 +77,41 @@ def test_a_batch_is_the_sum_of_its_parts(shape):
     for a, b in zip(whole, parts):
         assert np.abs(b).max() > 0
         assert np.abs(a - b).max() <= 1e-4 * np.abs(b).max()
+
+
+@pytest.mark.parametrize("shape", [(16, 2, 64, 2, 18, 4, 0), (8, 2, 64, 1, 18, 2, 1), (16, 4, 128, 2, 18, 4, 0),
+                                   (4, 4, 128, 3, 10, 2, 0)])
+@pytest.mark.parametrize("n,live", [(4999, 3000), (4608, 128), (4481, 1), (4480, 0)])
+def test_rays_without_a_segment_change_nothing(shape, n, live):
+    """The first layer's kernels take rays in order of their segment count and leave tiles without one out: a batch
+    with rays that miss the box scattered through it against its other rays alone. Same products, sums in another
+    order: the bound of the test above. No other ray at all: no loss, no gradient."""
+    cfg, mesh, p = _object(*shape, N_max=12)
+    rays = torch.from_numpy(I.rays_sphere_to_box(4 * n, 2.0, mesh.verts.min(0), mesh.verts.max(0), 7)).cuda()
+    g = torch.Generator("cuda").manual_seed(2)
+    r = lambda *s: torch.rand(s, device="cuda", generator=g)  # noqa: E731
+    lab = {"occ": (r(n) < 0.7).float(), "t_local": r(n),
+           "normal": torch.nn.functional.normalize(r(n, 3) - 0.5, dim=1).contiguous(), "albedo": r(n, 3),
+           "mat": torch.randint(0, cfg.n_mat, (n,), device="cuda", generator=g, dtype=torch.int32)}
+    with lsnif.Context(0) as ctx:
+        obj = ctx.load_object(mesh, cfg, tables=p.tables, mlp=p.packed_mlp())
+        rays = rays[:, ctx.trace(rays, obj)[0] > 0][:, :n].contiguous()
+        assert rays.shape[1] == n
+        keep = torch.zeros(n, dtype=torch.bool, device="cuda")
+        keep[torch.randperm(n, device="cuda", generator=g)[:live]] = True
+        rays[:3, ~keep] += 1000.0  # far outside, pointing past the box
+        got = []
+        for sel in (slice(None), keep):
+            part = rays[:, sel].contiguous()
+            if part.shape[1] == 0:
+                continue
+            st = ctx.train_step(part, {a: v[sel].contiguous() for a, v in lab.items()}, obj, apply_update=False)
+            ctx.check()
+            got.append((np.float64(st.total), ctx.read_params(obj, lsnif.PARAM_GRAD_TABLES),
+                        ctx.read_params(obj, lsnif.PARAM_GRAD_MLP)))
+    if live == 0:
+        assert all(np.abs(x).max() == 0 for x in got[0])
+        return
+    for a, b in zip(*got):
+        assert np.abs(b).max() > 0
+        assert np.abs(a - b).max() <= 1e-4 * np.abs(b).max()
