@@ -277,6 +277,11 @@ cudaError_t launch_input_scatter(const DevObject *dobj, const DevObject &h, int6
                                  const void *w0t, const int32_t *k, const int32_t *order, const float *pts,
                                  float *gtab, float *dense, int *err, cudaStream_t st);
 
+// Weight and bias gradients (gW[l], gb[l]) of layers 1 .. n_hidden from the chain's
+// outputs (train_grads.cu). k: rows' segment counts where they fall, else NULL
+cudaError_t launch_layer_grads(const DevObject &h, int64_t B, const int32_t *k, const float *acts, const float *grads,
+                               const float *dZ, float *const *gW, float *const *gb, int *err, cudaStream_t st);
+
 // The first layer over rays in order of their segment count (train_layer0.cu):
 // row -> ray and segment count; features as tiles of two-term BF16 operands
 // (whole tiles of kTileM rows); forward product; weight and bias gradients

@@ -489,14 +489,25 @@ __global__ void widen_count_kernel(const uint8_t *k8, int64_t B, int32_t *k, flo
 
 __global__ void adam_kernel(float *p, const float *g, float *m, float *v, int64_t n, float lr, float b1, float b2,
                             float eps, float c1, float c2) {
-  for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-    const float gi = g[i];
-    const float mi = b1 * m[i] + (1.f - b1) * gi;
-    const float vi = b2 * v[i] + (1.f - b2) * gi * gi;
-    m[i] = mi;
-    v[i] = vi;
-    p[i] -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  auto one = [&](float &pi, float gi, float &mi, float &vi) {
+    mi = b1 * mi + (1.f - b1) * gi;
+    vi = b2 * vi + (1.f - b2) * gi * gi;
+    pi -= lr * (mi / c1) / (sqrtf(vi / c2) + eps);
+  };
+  const int64_t first = (int64_t)blockIdx.x * blockDim.x + threadIdx.x, step = (int64_t)gridDim.x * blockDim.x;
+  for (int64_t q = first; q < n / 4; q += step) {
+    float4 P = reinterpret_cast<float4 *>(p)[q], M = reinterpret_cast<float4 *>(m)[q],
+           Q = reinterpret_cast<float4 *>(v)[q];
+    const float4 G = reinterpret_cast<const float4 *>(g)[q];
+    one(P.x, G.x, M.x, Q.x);
+    one(P.y, G.y, M.y, Q.y);
+    one(P.z, G.z, M.z, Q.z);
+    one(P.w, G.w, M.w, Q.w);
+    reinterpret_cast<float4 *>(p)[q] = P;
+    reinterpret_cast<float4 *>(m)[q] = M;
+    reinterpret_cast<float4 *>(v)[q] = Q;
   }
+  for (int64_t i = (n & ~int64_t(3)) + first; i < n; i += step) one(p[i], g[i], m[i], v[i]);
 }
 
 }  // namespace
@@ -638,7 +649,12 @@ cudaError_t launch_train_step(const DevObject *objs, int n_slots, const DevObjec
     const int fi = l == 0 ? NI : W;
     const float *hin = l == 0 ? tb.feats : tb.acts + (size_t)(l - 1) * B * W;
     // dW = d^T . hin  (dcols x fi), split over the batch, and db
-    if (l == 0 && own) {
+    if (chain && l > 0) {  // all of them at once
+      if (l == NH) {
+        e = launch_layer_grads(h, B, own ? tb.k : nullptr, tb.acts, tb.pre, tb.dZ, gW, gb, err, st);
+        if (e != cudaSuccess) return e;
+      }
+    } else if (l == 0 && own) {
       e = launch_layer0_grad(dobj, h, B, tb.k, tb.feats, d, gW[0], gb[0], err, st);
       if (e != cudaSuccess) return e;
     } else {
