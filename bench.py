@@ -37,7 +37,8 @@ WORKLOAD = ("noise torus 200k tris; V=128^3; hash grid L=16 F=2 T=2^19 N=16..204
             "MLP 576-64x4-12; 2048x2048 pinhole primary rays")
 PROFILE_MD = os.path.join(ROOT, "profiles", "fused_kernel_torus_4m.md")
 FUSED_SOURCES = ["paper_2504_21627_gb300/csrc/fused.cu", "paper_2504_21627_gb300/csrc/encode.cuh",
-                 "paper_2504_21627_gb300/csrc/device.cuh", "paper_2504_21627_gb300/csrc/tc_common.cuh"]
+                 "paper_2504_21627_gb300/csrc/device.cuh", "paper_2504_21627_gb300/csrc/tc_common.cuh",
+                 "paper_2504_21627_gb300/csrc/tile_feed.cuh"]
 
 
 def fused_source_hash() -> str:
