@@ -160,7 +160,7 @@ extern "C" int lsnif_query_rays_noalloc(lsnif_ctx *ctx, const lsnif_rays *r, lsn
   q.group_mode = ctx->group_mode == 2 ? 3 : ctx->group_mode == 1 ? (r->obj ? 2 : 1) : 0;
   q.single_slot = r->obj ? 0 : rep->slot;
   // The bucket counts must start at zero: launch_trace clears them on the
-  // stream; the grouping kernel resets the cursors and the tile counter.
+  // stream; the cursors with them, or in the grouping, which resets the tile counter.
   int launches = 0;
   cudaError_t e = launch_trace(q, &launches);
   if (e == cudaSuccess) e = launch_group(q, &launches);

@@ -200,6 +200,7 @@ __global__ void __launch_bounds__(256) presort_scatter_kernel(QueryLaunch q) {
 // lane-by-lane refill) and this one: a million rays from a sphere 574 -> 333 us, a million from the
 // surface 335 -> 199 us, 4,096 rays 85 -> 48 us, 4.19M camera rays 588 -> 593 us.
 // ---------------------------------------------------------------------------
+constexpr int kOnceObjects = 32;  // group_at_once_kernel
 constexpr int kQueueWords = 14;  // words of a started ray in the queue
 constexpr int kShortRound = 16, kLongRound = 256;  // cells between two refills of a warp's idle lanes
 constexpr int kTraceWarps = 4;
@@ -524,33 +525,11 @@ __device__ __forceinline__ int tile_shift(int n_live, int sms) {
   return c2 < c1 && c2 < c0 ? 2 : (c1 < c0 ? 1 : 0);
 }
 
-// Single block: bucket offsets (object ascending, k descending), tiles of
-// kTileM rays that never straddle objects, totals, cursors reset. A warp takes
-// one object's 32 buckets at a time, so an object's range starts at the value
-// its lane 0 scans to. One thread walking the buckets (a load per bucket, none
-// in flight beside another) took 9.8 us on six objects; this takes 5.2.
-__global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
-  __shared__ int ws[33];
-  __shared__ int first[kMaxObjects + 1];     // start of each object's range
-  __shared__ int tile_off[kMaxObjects + 1];  // and its first tile
+// A block of 1024: totals and the tile table from the objects' ranges in the
+// order. first[s]: start of object s (the end of the last is set here); pts:
+// this thread's share of the point count; tile_off, ws: shared scratch.
+__device__ __forceinline__ void write_tiles(const QueryLaunch &q, int run, int pts, int *first, int *tile_off, int *ws) {
   const int ns = q.n_slots;
-  static_assert(kMaxCap == 32, "a warp per object");
-  int run = 0, pts = 0;
-  for (int base = 0; base < ns * kMaxCap; base += 1024) {
-    const int s = (base + (int)threadIdx.x) >> 5, k = kMaxCap - (threadIdx.x & 31);
-    const int c = s < ns ? q.s.counts[s * kBuckets + k] : 0;
-    int total;
-    const int at = run + block_scan(c, ws, total);
-    // group modes 2 and 3: one bucket per object (bucket k = 1 takes all)
-    const int start = __shfl_sync(0xffffffffu, at, 0);
-    if (s < ns) {
-      q.s.offsets[s * kBuckets + k] = q.group_mode >= 2 ? start : at;
-      q.s.cursor[s * kBuckets + k] = 0;
-      if (k == kMaxCap) first[s] = at;
-    }
-    pts += 2 * k * c;
-    run += total;
-  }
   int points;
   block_scan(pts, ws, points);  // also a barrier: first[] is written
   if (threadIdx.x == 0) first[ns] = run;
@@ -583,6 +562,36 @@ __global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
     q.s.tiles[3 * t + 1] = start;
     q.s.tiles[3 * t + 2] = min(kTileM, first[lo + 1] - start);
   }
+}
+
+// Single block: bucket offsets (object ascending, k descending), tiles of
+// kTileM rays that never straddle objects, totals, cursors reset. A warp takes
+// one object's 32 buckets at a time, so an object's range starts at the value
+// its lane 0 scans to. One thread walking the buckets (a load per bucket, none
+// in flight beside another) took 9.8 us on six objects; this takes 5.2.
+__global__ void __launch_bounds__(1024) scan_kernel(QueryLaunch q) {
+  __shared__ int ws[33];
+  __shared__ int first[kMaxObjects + 1];     // start of each object's range
+  __shared__ int tile_off[kMaxObjects + 1];  // and its first tile
+  const int ns = q.n_slots;
+  static_assert(kMaxCap == 32, "a warp per object");
+  int run = 0, pts = 0;
+  for (int base = 0; base < ns * kMaxCap; base += 1024) {
+    const int s = (base + (int)threadIdx.x) >> 5, k = kMaxCap - (threadIdx.x & 31);
+    const int c = s < ns ? q.s.counts[s * kBuckets + k] : 0;
+    int total;
+    const int at = run + block_scan(c, ws, total);
+    // group modes 2 and 3: one bucket per object (bucket k = 1 takes all)
+    const int start = __shfl_sync(0xffffffffu, at, 0);
+    if (s < ns) {
+      q.s.offsets[s * kBuckets + k] = q.group_mode >= 2 ? start : at;
+      q.s.cursor[s * kBuckets + k] = 0;
+      if (k == kMaxCap) first[s] = at;
+    }
+    pts += 2 * k * c;
+    run += total;
+  }
+  write_tiles(q, run, pts, first, tile_off, ws);
 }
 
 // Scatter live rays into their bucket ranges; warp-aggregated atomics keep
@@ -648,6 +657,53 @@ __global__ void __launch_bounds__(1024) scatter_block_kernel(QueryLaunch q, int 
   }
   __syncthreads();
   if (bucket >= 0) q.s.order[q.s.offsets[bucket] + s_base[bucket] + rank] = (int32_t)i;
+}
+
+// scan_kernel and scatter_block_kernel in one launch, for at most 32 objects:
+// every block scans the few counts itself, the first one writes the totals and
+// the tile table. The cursors were cleared with the counts (group_at_once).
+// Both launches against this one, between events: 4,096 to 100,000 rays 10.9 ->
+// 8.8 us, 300,000 14.5 -> 8.9, a million 22.7 -> 17.5, 4.19M 37.5 -> 31.3; the
+// query of 4,096 icosphere rays 57.2 -> 54.5 us. More objects than a block's
+// 1,024 threads have buckets for take the two launches.
+__global__ void __launch_bounds__(1024) group_at_once_kernel(QueryLaunch q) {
+  constexpr int NB = kOnceObjects * kBuckets;
+  __shared__ int ws[33], first[kOnceObjects + 1], tile_off[kOnceObjects + 1], s_cnt[NB], s_base[NB];
+  const int ns = q.n_slots, tid = threadIdx.x, lane = tid & 31;
+  const int64_t i = (int64_t)blockIdx.x * blockDim.x + tid;
+  int bucket = -1;
+  if (i < q.rays.n) {
+    const int k = q.s.k[i];
+    const int s = q.s.slot[i];
+    if (k > 0 && s >= 0) bucket = s * kBuckets + (q.group_mode == 2 ? 1 : k);
+  }
+  static_assert(kMaxCap == 32 && kOnceObjects * kMaxCap == 1024, "a warp per object, all objects at once");
+  const int so = tid >> 5, k = kMaxCap - lane;
+  const int c = so < ns ? q.s.counts[so * kBuckets + k] : 0;
+  for (int b = tid; b < ns * kBuckets; b += blockDim.x) s_cnt[b] = 0;
+  int run;
+  const int at = block_scan(c, ws, run);
+  const int start = __shfl_sync(0xffffffffu, at, 0);
+  if (so < ns) {
+    s_base[so * kBuckets + k] = q.group_mode >= 2 ? start : at;
+    if (lane == 0) first[so] = at;
+  }
+  const unsigned active = __ballot_sync(0xffffffffu, bucket >= 0);
+  int rank = 0;
+  if (bucket >= 0) {
+    const unsigned peers = __match_any_sync(active, bucket);
+    const int leader = __ffs(peers) - 1;
+    int wbase = 0;
+    if (lane == leader) wbase = atomicAdd(&s_cnt[bucket], __popc(peers));
+    wbase = __shfl_sync(peers, wbase, leader);
+    rank = wbase + __popc(peers & ((1u << lane) - 1u));
+  }
+  __syncthreads();
+  for (int b = tid; b < ns * kBuckets; b += blockDim.x)
+    if (s_cnt[b]) s_base[b] += atomicAdd(&q.s.cursor[b], s_cnt[b]);
+  __syncthreads();
+  if (bucket >= 0) q.s.order[s_base[bucket] + rank] = (int32_t)i;
+  if (blockIdx.x == 0) write_tiles(q, run, 2 * k * c, first, tile_off, ws);
 }
 
 // ---------------------------------------------------------------------------
@@ -1071,12 +1127,20 @@ static int trace_pool_share(int64_t n, int grid) {
   return 32 * (int)std::max<int64_t>(1, std::min<int64_t>(8, n / ((int64_t)grid * kTraceWarps * 32 * 8)));
 }
 
+// The counters, the histogram and the cursors lie together in the queries'
+// scratch and are cleared in one operation, up to the cursors where the
+// grouping at once needs them cleared.
+static bool group_at_once(const QueryLaunch &q) {
+  return q.s.counts == q.s.meta + kMetaWords && q.s.cursor > q.s.counts && q.s.cursor - q.s.meta < (1 << 14) &&
+         q.group_mode != 1 && q.group_mode != 3 && q.n_slots <= kOnceObjects;
+}
+
 cudaError_t launch_trace(const QueryLaunch &q, int *launches) {
   const int nb = q.n_slots * kBuckets;
   // the counters and the histogram, in one operation where they lie together
   const bool joined = q.s.counts == q.s.meta + kMetaWords;
-  cudaError_t e0 = cudaMemsetAsync(joined ? q.s.meta : q.s.counts, 0,
-                                   sizeof(int32_t) * (nb + (joined ? kMetaWords : 0)), q.stream);
+  const size_t words = group_at_once(q) ? q.s.cursor - q.s.meta + nb : nb + (joined ? kMetaWords : 0);
+  cudaError_t e0 = cudaMemsetAsync(joined ? q.s.meta : q.s.counts, 0, sizeof(int32_t) * words, q.stream);
   if (e0 == cudaSuccess && !joined) e0 = cudaMemsetAsync(q.s.meta + 4, 0, sizeof(int32_t), q.stream);
   if (e0 != cudaSuccess) return e0;
   const int smem_hist = nb <= 12288;
@@ -1141,6 +1205,11 @@ cudaError_t launch_group(const QueryLaunch &q, int *launches) {
     if (e != cudaSuccess) return e;
     spatial_scatter_kernel<<<blocks, 256, 0, q.stream>>>(q, bits);
     *launches += 6;
+    return cudaGetLastError();
+  }
+  if (group_at_once(q)) {
+    group_at_once_kernel<<<(unsigned)std::max<int64_t>((q.rays.n + 1023) / 1024, 1), 1024, 0, q.stream>>>(q);
+    *launches += 1;
     return cudaGetLastError();
   }
   scan_kernel<<<1, 1024, 0, q.stream>>>(q);
