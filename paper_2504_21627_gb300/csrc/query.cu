@@ -349,7 +349,10 @@ __global__ void __launch_bounds__(kTraceWarps * 32, kTraceCtas)
             cc = min(max(cc, 0), V - 1);
             if (a == ea) cc = dd[a] > 0.f ? 0 : V - 1;
             cell |= (uint32_t)cc << (10 * a);
-            near = near && (__reduce_max_sync(m, cc) - __reduce_min_sync(m, cc)) * 8 <= V;
+            // every live lane joins both reductions: V, and with it the verdict,
+            // differs between the lanes of a batch that mixes grids
+            const int span = __reduce_max_sync(m, cc) - __reduce_min_sync(m, cc);
+            near = near & (span * 8 <= V);
             sq[a][e] = __float_as_uint(oo[a]);
             sq[3 + a][e] = __float_as_uint(dd[a]);
             sq[6 + a][e] = __float_as_uint(dd[a] != 0.f ? 1.f / dd[a] : 0.f);
