@@ -454,9 +454,10 @@ LSNIF_API int lsnif_mlp(lsnif_ctx *ctx, lsnif_obj obj, const float *X, int64_t n
  * handle, fused-kernel variant and number of object slots -- into a CUDA
  * graph the first time and replays that graph afterwards (one launch instead
  * of the query's kernel sequence). Object parameters may change between
- * replays (kernels read them at run time). Graphs are dropped when the
- * scratch is reallocated or graph mode is switched off. Queries on the
- * legacy default stream, and profiled queries, run without graphs. */
+ * replays (kernels read them at run time). Graphs are dropped when an object
+ * is loaded or unloaded, when the scratch is reallocated and when graph mode
+ * is switched off. Queries on the legacy default stream, and profiled
+ * queries, run without graphs. */
 LSNIF_API int lsnif_set_graph_mode(lsnif_ctx *ctx, int on);
 
 /* ---- autotuning of the fused kernel's shape ----------------------------- */

@@ -554,6 +554,7 @@ static int load_mesh_object(lsnif_ctx *ctx, const lsnif_object_desc *desc, lsnif
   if (e == cudaSuccess) e = cudaMemcpy(ctx->d_objs + slot, &d, sizeof d, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { free_object(ctx, o); return cuda_fail(e, "lsnif_load_object: upload mesh object"); }
+  clear_graphs(ctx);
   ctx->n_slots_used = std::max(ctx->n_slots_used, slot + 1);
   *out = o->handle;
   return LSNIF_OK;
@@ -766,6 +767,7 @@ extern "C" int lsnif_load_object(lsnif_ctx *ctx, const lsnif_object_desc *desc, 
   e = cudaMemcpy(ctx->d_objs + slot, &d, sizeof d, cudaMemcpyHostToDevice);
   if (e == cudaSuccess) e = cudaDeviceSynchronize();
   if (e != cudaSuccess) { free_object(ctx, o); return cuda_fail(e, "lsnif_load_object: upload"); }
+  clear_graphs(ctx);  // their launches were chosen for the objects of their capture
   ctx->n_slots_used = std::max(ctx->n_slots_used, slot + 1);
   *out = o->handle;
   return LSNIF_OK;
@@ -782,6 +784,7 @@ extern "C" int lsnif_unload_object(lsnif_ctx *ctx, lsnif_obj h) {
   if (!o) return fail(LSNIF_ERR_BAD_HANDLE, "lsnif_unload_object: bad handle %u", h);
   cudaSetDevice(ctx->device);
   cudaDeviceSynchronize();
+  clear_graphs(ctx);
   free_object(ctx, o);
   return LSNIF_OK;
 }

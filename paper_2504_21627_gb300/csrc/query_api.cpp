@@ -278,8 +278,10 @@ void lsnif::clear_graphs(lsnif_ctx *ctx) {
 }
 
 // Replay a captured graph of this exact query, capturing it first. The key
-// holds everything the launch sequence depends on; the scratch must already
-// be large enough so that nothing is allocated while capturing.
+// holds what the launch sequence depends on apart from the set of objects
+// (kernels, template arguments and shared-memory sizes follow their shapes):
+// loading or unloading one drops every graph. The scratch must already be
+// large enough so that nothing is allocated while capturing.
 static int query_graph(lsnif_ctx *ctx, const lsnif_rays *r, lsnif_hits *h, int precision, cudaStream_t st) {
   int rc = check_rays(r, h);
   if (rc) return rc;
