@@ -709,13 +709,10 @@ static int pick_nbuf(const DevObject &h, int list_chunks, bool fp16) {
 
 template <int F, int W, bool XR, int NG, int NLB, int GS, bool H16>
 static cudaError_t launch_op(const FusedArgs &a, size_t smem, cudaStream_t st) {
-  static int attr = 0;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(fused_kernel<F, W, XR, NG, NLB, GS, H16>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = 1;
-  }
+  // on every launch: the limit belongs to the current device
+  const cudaError_t e = cudaFuncSetAttribute(fused_kernel<F, W, XR, NG, NLB, GS, H16>,
+                                             cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

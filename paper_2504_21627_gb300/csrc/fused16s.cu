@@ -557,13 +557,10 @@ size_t fused16s_smem_bytes(const DevObject &h, int H_max) {
 
 template <int F, int W, int NG, int NL>
 static cudaError_t launch16s_shape(const Fused16sArgs &a, size_t smem, cudaStream_t st) {
-  static int attr = 0;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(fused16s_kernel<F, W, NG, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = 1;
-  }
+  // on every launch: the limit belongs to the current device
+  const cudaError_t e =
+      cudaFuncSetAttribute(fused16s_kernel<F, W, NG, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

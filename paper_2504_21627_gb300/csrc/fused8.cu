@@ -684,13 +684,10 @@ constexpr int kNumVariants8 = (int)(sizeof(kVariants8) / sizeof(kVariants8[0]));
 
 template <int F, int W, int NG, int NL>
 static cudaError_t launch8_shape(const Fused8Args &a, size_t smem, cudaStream_t st) {
-  static int attr = 0;
-  if (!attr) {
-    cudaError_t e =
-        cudaFuncSetAttribute(fused8_kernel<F, W, NG, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = 1;
-  }
+  // on every launch: the limit belongs to the current device
+  const cudaError_t e =
+      cudaFuncSetAttribute(fused8_kernel<F, W, NG, NL>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  if (e != cudaSuccess) return e;
   int sms = 0, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);

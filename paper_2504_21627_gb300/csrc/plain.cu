@@ -374,9 +374,10 @@ size_t plain_smem(int lf_max) {
 template <int F, int W, int R>
 cudaError_t launch_rows(const QueryLaunch &q, int lf_max, int sms) {
   const size_t smem = plain_smem<W, R>(lf_max);
-  static const cudaError_t attr =
+  // on every launch: the limit belongs to the current device
+  const cudaError_t e =
       cudaFuncSetAttribute(plain_fused_kernel<F, W, R>, cudaFuncAttributeMaxDynamicSharedMemorySize, 96 << 10);
-  if (attr != cudaSuccess) return attr;
+  if (e != cudaSuccess) return e;
   const int64_t tiles = (int64_t)q.s.max_tiles * PlainShape<W, R>::SUB;
   const int grid = (int)std::max<int64_t>(1, std::min<int64_t>((int64_t)PlainShape<W, R>::CTAS * sms, tiles));
   plain_fused_kernel<F, W, R><<<grid, PlainShape<W, R>::T, smem, q.stream>>>(q, lf_max);

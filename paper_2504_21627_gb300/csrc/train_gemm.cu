@@ -362,17 +362,12 @@ cudaError_t launch_tc_gemm(cudaStream_t st, int M, int N, int K, const float *A,
   g.nst = g.k_per_z > kGK ? 2 : 1;
   // the stages (reused for a 128 x 33 piece of the product) + barriers + alignment slack
   const size_t smem = g.nst * stage + 64 + 1024;
-  static int attr = 0;
-  if (!attr) {
-    cudaError_t e = cudaFuncSetAttribute(tc_gemm_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e == cudaSuccess)
-      e = cudaFuncSetAttribute(tc_gemm_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
-    if (e != cudaSuccess) return e;
-    attr = 1;
-  }
+  // on every launch: the limit belongs to the current device
+  const auto kern = g.nst > 1 ? tc_gemm_kernel<true> : tc_gemm_kernel<false>;
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, 232448);
+  if (e != cudaSuccess) return e;
   dim3 grid((M + kGM - 1) / kGM, (N + g.n_ch - 1) / g.n_ch, nz);
-  if (g.nst > 1) tc_gemm_kernel<true><<<grid, kGThreads, smem, st>>>(g);
-  else tc_gemm_kernel<false><<<grid, kGThreads, smem, st>>>(g);
+  kern<<<grid, kGThreads, smem, st>>>(g);
   return cudaGetLastError();
 }
 
