@@ -1104,6 +1104,7 @@ __global__ void __launch_bounds__(256) mlp_fp32_rows_kernel(const DevObject *dob
   }
 }
 
+constexpr int kMlpSmemMax = 232448;  // all a CTA may have
 static size_t mlp_fp32_smem(int wmax) {
   return sizeof(float) * ((size_t)kKC * kMT + (size_t)kKC * wmax + 2 * (size_t)wmax * kMT);
 }
@@ -1239,7 +1240,8 @@ cudaError_t launch_exclusive_scan(int32_t *v, int64_t n, int32_t *sums, cudaStre
 
 cudaError_t launch_plain_tail(const QueryLaunch &q, int ldx, int chunk_tiles, int *launches) {
   const size_t smem = mlp_fp32_smem(q.s.wmax);
-  cudaError_t e = cudaFuncSetAttribute(mlp_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > kMlpSmemMax) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(mlp_fp32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
   if (e != cudaSuccess) return e;
   for (int t0 = 0; t0 < q.s.max_tiles; t0 += chunk_tiles) {
     const int nt = min(chunk_tiles, q.s.max_tiles - t0);
@@ -1349,7 +1351,8 @@ cudaError_t launch_mlp_plain(const DevObject *dobj, const DevObject &h, const fl
                              cudaStream_t st) {
   const int wmax = max(h.width, h.n_out_pad);
   const size_t smem = mlp_fp32_smem(wmax);
-  cudaError_t e = cudaFuncSetAttribute(mlp_fp32_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  if (smem > kMlpSmemMax) return cudaErrorInvalidValue;
+  cudaError_t e = cudaFuncSetAttribute(mlp_fp32_rows_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, kMlpSmemMax);
   if (e != cudaSuccess) return e;
   mlp_fp32_rows_kernel<<<grid_for(n, kMT, 152 * 4), 256, smem, st>>>(dobj, X, n, Z, wmax);
   return cudaGetLastError();

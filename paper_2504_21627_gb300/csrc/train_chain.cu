@@ -31,6 +31,7 @@ namespace lsnif {
 
 namespace {
 
+constexpr int kChainSmemMax = 200 << 10;  // dynamic shared memory of the largest network taken
 constexpr int kCThreads = 128;  // a thread per row; warp w has TMEM lane quarter w
 
 struct ChainArgs {
@@ -328,7 +329,7 @@ __global__ void __launch_bounds__(kCThreads) train_chain_kernel(const __grid_con
 
 template <int W, int NZ>
 cudaError_t launch_shape(const ChainArgs &a, size_t smem, cudaStream_t st) {
-  cudaError_t e = cudaFuncSetAttribute(train_chain_kernel<W, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  cudaError_t e = cudaFuncSetAttribute(train_chain_kernel<W, NZ>, cudaFuncAttributeMaxDynamicSharedMemorySize, kChainSmemMax);
   if (e != cudaSuccess) return e;
   int sms = 152, dev = 0;
   cudaGetDevice(&dev);
@@ -347,7 +348,7 @@ size_t chain_smem(const DevObject &h) {
 }  // namespace
 
 bool train_chain_supported(const DevObject &h) {
-  return (h.width == 64 || h.width == 128) && h.n_out_pad <= 64 && chain_smem(h) <= 200u * 1024u;
+  return (h.width == 64 || h.width == 128) && h.n_out_pad <= 64 && chain_smem(h) <= kChainSmemMax;
 }
 
 cudaError_t launch_train_chain(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k,

@@ -213,15 +213,15 @@ __global__ void __launch_bounds__(kGradThreads, W == 64 ? 3 : 1) layer_grads_ker
 
 template <int W>
 cudaError_t launch_shape(const GradArgs &a, cudaStream_t st) {
-  constexpr size_t smem = 4 * (size_t)kTileM * W * 2 + 1024;
-  const cudaError_t e = cudaFuncSetAttribute(layer_grads_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  constexpr int kSmem = 4 * kTileM * W * 2 + 1024;
+  const cudaError_t e = cudaFuncSetAttribute(layer_grads_kernel<W>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmem);
   if (e != cudaSuccess) return e;
   int sms = 152, dev = 0;
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   const int per_layer = std::max(1, sms * (W == 64 ? 3 : 1) / a.n_layers);
   const dim3 grid((unsigned)std::min<int64_t>(a.n_tiles, per_layer), (unsigned)a.n_layers);
-  layer_grads_kernel<W><<<grid, kGradThreads, smem, st>>>(a);
+  layer_grads_kernel<W><<<grid, kGradThreads, kSmem, st>>>(a);
   return cudaGetLastError();
 }
 

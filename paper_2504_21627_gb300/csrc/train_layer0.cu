@@ -520,7 +520,8 @@ int sm_count() {
   return sms;
 }
 
-constexpr size_t kSmemMax = 222u << 10;  // dynamic: the static part and the system's 1 KB come on top
+constexpr int kSmemMax = 222 << 10;  // dynamic: the static part and the system's 1 KB come on top
+constexpr int kSumBytes = 8192;     // the column sums (static, layer0_grad_kernel)
 
 Layer0Args layer0_args(const DevObject *dobj, const DevObject &h, int64_t B, const int32_t *k, const void *x) {
   Layer0Args a{};
@@ -566,7 +567,7 @@ cudaError_t launch_layer0(const DevObject *dobj, const DevObject &h, int64_t B, 
   const size_t smem = a.stages * stage + 1024;
   const unsigned grid = (unsigned)std::min<int64_t>(a.n_tiles, sm_count());
   auto *kern = h.width == 64 ? layer0_kernel<64> : layer0_kernel<128>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax);
   if (e != cudaSuccess) return e;
   kern<<<grid, kFwdThreads, smem, st>>>(a);
   return cudaGetLastError();
@@ -583,12 +584,12 @@ cudaError_t launch_layer0_grad(const DevObject *dobj, const DevObject &h, int64_
   int y = 1;
   while ((a.n_seg + y - 1) / y * a.chk > 512) ++y;
   const size_t stage = 4 * (size_t)a.chk * kTileM, yb = 8 * (size_t)kTileM * h.width + 1024;
-  const size_t room = kSmemMax - 8192 - 1024 - yb;  // 8 KB: the column sums
+  const size_t room = kSmemMax - kSumBytes - 1024 - yb;
   a.stages = (int)std::max<size_t>(1, std::min<size_t>(kMaxStages, room / stage));
   const size_t smem = a.stages * stage + yb + 1024;
   const dim3 grid((unsigned)std::min<int64_t>(a.n_tiles, std::max(1, sm_count() / y)), (unsigned)y);
   auto *kern = h.width == 64 ? layer0_grad_kernel<64> : layer0_grad_kernel<128>;
-  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  const cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemMax - kSumBytes);
   if (e != cudaSuccess) return e;
   kern<<<grid, kGradThreads, smem, st>>>(a);
   return cudaGetLastError();

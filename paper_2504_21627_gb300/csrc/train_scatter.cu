@@ -327,8 +327,10 @@ __global__ void __launch_bounds__(256) dense_sum_kernel(ScatterArgs a) {
 
 template <int F, int HC>
 cudaError_t launch_shape(const ScatterArgs &a, cudaStream_t st) {
-  const size_t smem = 2 * (size_t)kTileM * a.W * 2 + 4 * (size_t)(4 * HC) * a.W * 2 + 1024;
-  const cudaError_t e = cudaFuncSetAttribute(input_scatter_kernel<F, HC>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+  auto smem_of = [](int W) { return 2 * (size_t)kTileM * W * 2 + 4 * (size_t)(4 * HC) * W * 2 + 1024; };
+  const size_t smem = smem_of(a.W);
+  const cudaError_t e = cudaFuncSetAttribute(input_scatter_kernel<F, HC>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                             (int)smem_of(128));
   if (e != cudaSuccess) return e;
   input_scatter_kernel<F, HC><<<(unsigned)((a.B + kTileM - 1) / kTileM), kSThreads, smem, st>>>(a);
   return cudaGetLastError();

@@ -1,5 +1,6 @@
 """How the launchers raise a kernel's shared-memory limit, read from their sources (one GPU cannot show it): the limit
-belongs to the device that is current, so no launcher may raise it once per process only."""
+belongs to the device that is current, so no launcher may raise it once per process only; and it is shared by the
+threads that launch the kernel, so it is one bound for every call, not the size that this call needs."""
 import glob
 import os
 import re
@@ -31,3 +32,11 @@ def test_launchers_are_found():
 def test_the_limit_is_raised_on_every_launch(i):
     name, body = LAUNCHERS[i]
     assert not re.search(r"\bstatic\s+(const\s+)?\w+(\s+\w+|\s*<[^>]*>\s*\w+)\s*[=;{]", body), f"{name}: kept between calls:\n{body}"
+
+
+@pytest.mark.parametrize("i", range(len(LAUNCHERS)))
+def test_the_limit_is_the_same_in_every_call(i):
+    name, body = LAUNCHERS[i]
+    for call in re.findall(r"cudaFuncSetAttribute\((?:[^()]|\([^()]*\))*\)", body):
+        limit = call.split("cudaFuncAttributeMaxDynamicSharedMemorySize,")[1]
+        assert not re.search(r"\bsmem\b", limit), f"{name}: {call}"
