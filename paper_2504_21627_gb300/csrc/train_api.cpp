@@ -4,6 +4,8 @@
 
 #include <algorithm>
 #include <cstring>
+#include <utility>
+#include <vector>
 
 #include "lsnif_impl.h"
 #include "runtime.h"
@@ -19,7 +21,7 @@ void lsnif::free_train_state(lsnif_ctx *ctx, Object *o) {
 }
 
 void lsnif::reset_optimizer(lsnif_ctx *, Object *o) {
-  if (!o->tb.m_mlp) return;
+  if (!o->tb.v_tab) return;  // the last of the state to be allocated: no step has used it yet
   const lsnif_config &c = o->cfg;
   const size_t nt = ((size_t)c.L << c.log2_T) * c.F;
   cudaMemset(o->tb.m_mlp, 0, 4 * o->n_params_mlp);
@@ -35,14 +37,23 @@ static int train_alloc(lsnif_ctx *ctx, Object *o, size_t bytes, void **p, const 
   return rc;
 }
 
-// Size the batch buffers for B rays; the optimiser state survives regrowth.
+// Size the batch buffers for B rays; the optimiser state and the gradients
+// survive regrowth. After a failure the object has no batch buffers (the next
+// step allocates them again) and keeps what it has of the rest.
 static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
   if (o->tb_batch >= B && o->tb.feats) return LSNIF_OK;
   cudaDeviceSynchronize();
   const lsnif_config &c = o->cfg;
   const size_t nt = ((size_t)c.L << c.log2_T) * c.F;
-  TrainBuffers keep = o->tb;
-  // batch-sized buffers are reallocated; optimiser state and gradients kept
+  TrainBuffers &tb = o->tb;
+  TrainBuffers keep{};
+  keep.loss = tb.loss;
+  keep.grad_mlp = tb.grad_mlp;
+  keep.grad_tab = tb.grad_tab;
+  keep.m_mlp = tb.m_mlp;
+  keep.v_mlp = tb.v_mlp;
+  keep.m_tab = tb.m_tab;
+  keep.v_tab = tb.v_tab;
   std::vector<void *> persistent;
   for (void *p : o->train_allocs) {
     if (p == keep.m_mlp || p == keep.v_mlp || p == keep.m_tab || p == keep.v_tab || p == keep.grad_mlp ||
@@ -52,7 +63,8 @@ static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
       dev_free(ctx, p);
   }
   o->train_allocs = persistent;
-  TrainBuffers &tb = o->tb;
+  tb = keep;
+  o->tb_batch = 0;
   const int W = c.width, NI = o->d.n_in, NO = o->d.n_out;
   void *p;
   int rc;
@@ -75,9 +87,6 @@ static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
   TALLOC(dZ, float *, 4 * (size_t)B * NO);
   TALLOC(dA, float *, 4 * (size_t)B * W);
   TALLOC(dB, float *, 4 * (size_t)B * W);
-  tb.w0t = nullptr;
-  tb.dense = nullptr;
-  tb.order = nullptr;
   if (own) {
     TALLOC(order, int32_t *, order_bytes);
     TALLOC(w0t, void *, plan.w0t_bytes);
@@ -91,30 +100,18 @@ static int ensure_train(lsnif_ctx *ctx, Object *o, int64_t B) {
   TALLOC(slot, int16_t *, 2 * (size_t)B);
   TALLOC(counts, int32_t *, 4 * (size_t)kMaxSlots * kBuckets);
   TALLOC(meta, int32_t *, 64);
-  if (!keep.loss) {
-    TALLOC(loss, float *, 64);
-    TALLOC(grad_mlp, float *, 4 * (size_t)o->n_params_mlp);
-    TALLOC(grad_tab, float *, 4 * nt);
-    TALLOC(m_mlp, float *, 4 * (size_t)o->n_params_mlp);
-    TALLOC(v_mlp, float *, 4 * (size_t)o->n_params_mlp);
-    TALLOC(m_tab, float *, 4 * nt);
-    TALLOC(v_tab, float *, 4 * nt);
-    cudaMemset(tb.m_mlp, 0, 4 * o->n_params_mlp);
-    cudaMemset(tb.v_mlp, 0, 4 * o->n_params_mlp);
-    cudaMemset(tb.m_tab, 0, 4 * nt);
-    cudaMemset(tb.v_tab, 0, 4 * nt);
-    cudaMemset(tb.grad_mlp, 0, 4 * o->n_params_mlp);
-    cudaMemset(tb.grad_tab, 0, 4 * nt);
-  } else {
-    tb.loss = keep.loss;
-    tb.grad_mlp = keep.grad_mlp;
-    tb.grad_tab = keep.grad_tab;
-    tb.m_mlp = keep.m_mlp;
-    tb.v_mlp = keep.v_mlp;
-    tb.m_tab = keep.m_tab;
-    tb.v_tab = keep.v_tab;
-  }
 #undef TALLOC
+  // what outlives a regrowth, each from the first time it can be had
+  const size_t mlp_bytes = 4 * (size_t)o->n_params_mlp, tab_bytes = 4 * nt;
+  const std::pair<float **, size_t> lasting[] = {{&tb.loss, 64},           {&tb.grad_mlp, mlp_bytes}, {&tb.grad_tab, tab_bytes},
+                                                 {&tb.m_mlp, mlp_bytes},   {&tb.v_mlp, mlp_bytes},    {&tb.m_tab, tab_bytes},
+                                                 {&tb.v_tab, tab_bytes}};
+  for (auto [field, bytes] : lasting) {
+    if (*field) continue;
+    if ((rc = train_alloc(ctx, o, bytes, &p, "training buffers")) != LSNIF_OK) return rc;
+    *field = (float *)p;
+    cudaMemset(p, 0, bytes);
+  }
   o->tb_batch = B;
   return LSNIF_OK;
 }
