@@ -683,9 +683,20 @@ bool fused_supported(const DevObject &h) {
 static uint32_t blob_bytes(const DevObject &h) { return (h.umma_bytes + 15u) & ~15u; }
 static uint32_t lo_bytes(const DevObject &h, bool fp16) { return fp16 ? 0u : (h.umma_lo_bytes + 15u) & ~15u; }
 
-// with the smallest ring (2 buffers); launches use up to kNBufMax that fit
+// The size by which queries choose this kernel: its shared memory with the
+// smallest ring (2 buffers; launches use up to kNBufMax that fit), with two
+// tiles' entry and exit times and two words per warp and chunk counted in place
+// of the masks. The line is drawn there and not at what the layout takes
+// (`held` bytes less) because it decides how an FP16 query rounds: the streamed
+// kernel interpolates features in FP32, this one's F = 2 gather in FP16. A
+// network on the other side of it would lose precision; in the 1.7 KB between
+// (16 levels x 2, 2 x 128 in FP16) it would also be slower on rays in no order:
+// 262,144 sphere rays 1134 us streamed, 1416 us here, although camera frames
+// are faster here (4.19M: 7257 and 4184 us).
 size_t fused_smem_bytes(const DevObject &h, int H_max, bool fp16) {
-  return make_layout(blob_bytes(h), lo_bytes(h, fp16), h.F, h.width, 2, std::max(H_max, h.H) / 2).total;
+  const int chunks = std::max(H_max, h.H) / 2;
+  const uint32_t held = 2 * 2 * kTileM * 4 - 32 * chunks - (8 * chunks + 15) / 16 * 16;
+  return make_layout(blob_bytes(h), lo_bytes(h, fp16), h.F, h.width, 2, chunks).total + held;
 }
 
 // Shared memory and L1 share one array per SM. A CTA that needs more than
