@@ -16,8 +16,8 @@
 // Warp roles:
 //   gather warps (NG): fill chunk after chunk into a ring of shared-memory A
 //     tiles;
-//   one MMA warp: issues each filled chunk's MMAs against the resident
-//     first-layer weights into the tile's TMEM accumulator;
+//   one MMA warp: copies shared points, issues each filled chunk's MMAs against
+//     the resident first-layer weights into the tile's TMEM accumulator;
 //   four epilogue warps (TMEM lane = ray): set the next tile up (rows, work
 //     lists), then hidden and output layers (bias, activation, 16-bit
 //     activations back to tensor memory, next MMA) and the decode, while the
@@ -29,15 +29,20 @@
 // for them. Shared boundary points: consecutive occupied voxels along a ray
 // share a face, and the traversal marks an entry point that is bit-identical
 // to the previous segment's exit (bit s of the ray's dup mask). Such a point
-// is gathered once: the MMAs of its chunk's entry half read the previous
-// chunk's exit half for the marked rows, and this chunk's entry half for the
-// others. Each row sees the same products in the same order as if its
-// features had been copied and its empty segments filled with zeros, as an
-// earlier form did with a quarter of the gather warps' time (the fused kernel
-// of 4.19M camera rays 2.32 -> 2.03 ms, of a million secondary rays 1.41 ->
-// 1.27 ms). Gathers go round-robin over the gather warps in blocks of 32 items
-// (item = one point x one 16-byte column group), so every warp gets the same
-// share.
+// is gathered once: the MMA warp copies its features from the previous chunk's
+// tile before it multiplies, which leaves the gather warps to their loads (an
+// earlier form copied and zero-filled with a quarter of their time: the fused
+// kernel of 4.19M camera rays 2.32 -> 2.03 ms, of a million secondary rays
+// 1.41 -> 1.27 ms). MMAs that read the shared points in the previous chunk's
+// tile instead serve only L F = 0 modulo 16, since half a step of K cannot come
+// from another tile, take a third pass per chunk and keep that tile's slot
+// longer. 4.19M rays, so (the points gathered twice where L F = 8 modulo 16)
+// and copied: 12 levels x 2, 4 x 64 from a sphere 11.17 and 8.88 ms, 16 x 4,
+// 1 x 64 (a ring of two slots) from the surface 10.19 and 9.77 ms, icosphere
+// network from the surface 3.83 and 3.76 ms (spatially grouped) and from a
+// sphere 4.62 and 4.67 ms, torus network within 0.6%. Gathers go round-robin
+// over the gather warps in blocks of 32 items (item = one point x one 16-byte
+// column group), so every warp gets the same share.
 //
 // Every mbarrier wait is bounded by a clock limit; on expiry the kernel flags
 // an abort, every role stops, the device error word is set, in-flight MMAs
@@ -167,6 +172,27 @@ __host__ __device__ inline Layout make_layout(uint32_t blob_bytes, uint32_t lo_b
 
 }  // namespace
 
+// A warp copies the exit points of `from` (a chunk's tile) to the entry points
+// of `to` in the rows given by the masks' second and fourth words (32 rows
+// each); G 16-byte groups per point.
+__device__ __forceinline__ void copy_shared(uint8_t *to, const uint8_t *from, const uint4 &m01, const uint4 &m23, int G,
+                                            uint32_t sbo, int lane) {
+  const bool d[4] = {((m01.y >> lane) & 1u) != 0u, ((m01.w >> lane) & 1u) != 0u, ((m23.y >> lane) & 1u) != 0u,
+                     ((m23.w >> lane) & 1u) != 0u};
+#pragma unroll 2
+  for (int g = 0; g < G; ++g) {
+    uint4 v[4];
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+      if (d[w]) v[w] = *reinterpret_cast<const uint4 *>(from + core_off(32 * w + lane, G + g, sbo));
+#pragma unroll
+    for (int w = 0; w < 4; ++w)
+      if (d[w]) *reinterpret_cast<uint4 *>(to + core_off(32 * w + lane, g, sbo)) = v[w];
+  }
+  fence_async_smem();
+  __syncwarp();
+}
+
 // The MMA warp's work (see epilogue_role for why it is a function).
 template <int F, int W, bool XROWS, int NG, bool H16>
 __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32_t tmem) {
@@ -189,20 +215,24 @@ __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32
     int rbuf = 0, ruse = 0;  // ring slot and pass of the next chunk
     int loads = 0;           // weight loads waited for
     const uint32_t idesc0 = idesc_f16(W, H16);
+    // a wait of the whole warp: the lanes go on, or give up, together
+    auto wait = [&](uint64_t *bar, uint32_t parity) {
+      return __all_sync(0xffffffffu, mbar_wait_sleep(su32(bar), parity, abort_flag)) != 0;
+    };
     for (int i = 0;; ++i) {
       const int tb = i & 1;
-      if (!mbar_wait_sleep(su32(&b_ready[tb]), (uint32_t)((i >> 1) & 1), abort_flag)) break;
+      if (!wait(&b_ready[tb], (uint32_t)((i >> 1) & 1))) break;
       const TileInfo ti = s_info[tb];
       if (ti.stop) break;
       if (ti.loads != loads) {  // this tile is the first with its object's weights
         loads = ti.loads;
-        if (!mbar_wait_sleep(su32(b_w), (uint32_t)((loads - 1) & 1), abort_flag)) break;
+        if (!wait(b_w, (uint32_t)((loads - 1) & 1))) break;
       }
       const DevObject &ob = objs[ti.slot];
       const int LF = ob.L * F, CHK = 2 * LF;
       const uint32_t a_sbo = (uint32_t)(CHK / 8) * 128u, w0_sbo = (uint32_t)(ob.n_in / 8) * 128u;
       const uint4 *masks = reinterpret_cast<const uint4 *>(base + lay.masks) + (size_t)tb * a.list_chunks * 2;
-      if (i >= 2 && !mbar_wait_sleep(su32(&b_acce[tb]), (uint32_t)(((i - 2) >> 1) & 1), abort_flag)) break;
+      if (i >= 2 && !wait(&b_acce[tb], (uint32_t)(((i - 2) >> 1) & 1))) break;
       tc_after();
       const uint32_t dacc = tmem + (uint32_t)(tb * W);
       bool ok = true;
@@ -216,35 +246,24 @@ __device__ __noinline__ void mma_role(const FusedArgs *ap, uint8_t *base, uint32
           rbuf = 0;
           ++ruse;
         }
-        if (!mbar_wait_sleep(su32(&b_full[buf]), phase, abort_flag)) {
+        if (!wait(&b_full[buf], phase)) {
           ok = false;
           break;
         }
         tc_after();
+        // (rows with a segment s, of those the shared entry points) of warps 0, 1 | 2, 3
+        const uint4 m01 = masks[2 * s], m23 = masks[2 * s + 1];
+        if (m01.y | m01.w | m23.y | m23.w)
+          copy_shared(s_ring + buf * ring_stride, s_ring + prev * ring_stride, m01, m23, LF / 8, a_sbo, lane);
         if (lane == 0) {
-          const uint32_t a0 = su32(s_ring + buf * ring_stride), ap = su32(s_ring + prev * ring_stride),
-                         b0 = su32(s_blob) + (uint32_t)((s * CHK) / 8) * 128u;
-          // (rows with a segment s, of those the shared entry points) of warps 0, 1 | 2, 3
-          const uint4 m01 = masks[2 * s], m23 = masks[2 * s + 1];
-          const uint4 off = make_uint4(~m01.x, ~m01.z, ~m23.x, ~m23.z);
-          auto multiply = [&](uint32_t at, uint32_t bt, int steps, const uint4 &o, bool first) {
-            for (int ks = 0; ks < steps; ++ks)
-              mma_f16_rows(dacc, umma_desc(at + ks * 256, 128, a_sbo), umma_desc(bt + ks * 256, 128, w0_sbo), idesc0, o,
-                           first && ks == 0 ? 0u : 1u);
-          };
-          if (LF % 16 == 0) {
-            const int h = LF / 16;  // steps of one point
-            // entry points: the chunk before holds the shared ones as its exit points
-            if (m01.y | m01.w | m23.y | m23.w)
-              multiply(ap + h * 256, b0, h, make_uint4(~m01.y, ~m01.w, ~m23.y, ~m23.w), false);
-            multiply(a0, b0, h, make_uint4(off.x | m01.y, off.y | m01.w, off.z | m23.y, off.w | m23.w), s == 0);
-            multiply(a0 + h * 256, b0 + h * 256, h, off, false);
-          } else {
-            multiply(a0, b0, CHK / 16, off, s == 0);
-          }
-          // the slot of the chunk before is free once these are done; the last
-          // chunk has no reader after it
+          // the slot of the chunk before is free once its own MMAs are done;
+          // the last chunk's shared points have no reader after it
           if (s > 0) mma_commit(su32(&b_empty[prev]));
+          const uint32_t a0 = su32(s_ring + buf * ring_stride), b0 = su32(s_blob) + (uint32_t)((s * CHK) / 8) * 128u;
+          const uint4 off = make_uint4(~m01.x, ~m01.z, ~m23.x, ~m23.z);
+          for (int ks = 0; ks < CHK / 16; ++ks)
+            mma_f16_rows(dacc, umma_desc(a0 + ks * 256, 128, a_sbo), umma_desc(b0 + ks * 256, 128, w0_sbo), idesc0, off,
+                         (s > 0 || ks > 0) ? 1u : 0u);
           if (s + 1 == ti.kmax) mma_commit(su32(&b_empty[buf]));
         }
         prev = buf;
@@ -328,10 +347,7 @@ __device__ __noinline__ void epilogue_role(const FusedArgs *ap, uint8_t *base, u
       if (etid < LSNIF_MAX_LEVELS) s_res[etid] = (float)ob.res[etid];
     }
     s_ray[sb * kTileM + etid] = feed.ray;
-    // a half step of K (L F = 8 mod 16) cannot be read from another chunk's
-    // tile: shared points are gathered twice then
-    const uint32_t dm = (objs[feed.slot].L * F) % 16 == 0 ? feed.dm : 0u;
-    const int kmax = build_lists<false>(etid, feed.kk, dm, s_list + (size_t)sb * a.list_chunks * kListStride,
+    const int kmax = build_lists<false>(etid, feed.kk, feed.dm, s_list + (size_t)sb * a.list_chunks * kListStride,
                                         s_masks + (size_t)sb * a.list_chunks * 4,
                                         s_counts + (size_t)sb * a.list_chunks, s_misc, a.list_chunks);
     named_sync(2, kFeedThreads);
@@ -469,7 +485,7 @@ __global__ void __launch_bounds__((NG + 1 + kEpiWarps) * 32, 1) fused_kernel(con
   uint64_t *b_accf = b_ready + 2, *b_acce = b_ready + 4, *b_layer = b_ready + 6, *b_fin = b_ready + 7;
   uint64_t *b_w = b_ready + 9;
   uint32_t *s_tmem = reinterpret_cast<uint32_t *>(base + lay.tmem);
-  int32_t *s_misc = reinterpret_cast<int32_t *>(base + lay.misc);  // [0] tile [1] kmax [2] epi stop [4] abort
+  int32_t *s_misc = reinterpret_cast<int32_t *>(base + lay.misc);  // [2] epilogue stop [4] abort [8..15] tile_feed.cuh
   volatile int *abort_flag = reinterpret_cast<volatile int *>(s_misc + 4);
   float *s_res = reinterpret_cast<float *>(base + lay.res);
   const uint32_t ring_stride = lay.ring_stride;
