@@ -355,8 +355,7 @@ __device__ __noinline__ void epilogue_role(const FusedArgs *ap, uint8_t *base, u
       s_info[sb].kmax = kmax;
       s_info[sb].slot = feed.slot;
       s_info[sb].stop = 0;
-      s_info[sb].rows = (int16_t)feed.cnt;
-      s_info[sb].loads = (int16_t)(loads & 0x7fff);
+      s_info[sb].loads = loads;
       mbar_arrive(su32(&b_ready[sb]));
     }
     feed.stage = 0;
@@ -719,11 +718,13 @@ size_t fused_smem_bytes(const DevObject &h, int H_max, bool fp16) {
 // the 196 KiB configuration (less the 1 KiB the system keeps per CTA) gets
 // the 228 KiB one, which leaves L1 28 KiB instead of 60 KiB; the gather's
 // coarse levels live in L1, and on the torus workload that alone took the
-// fused kernel from 2.79 to 3.93 ms. A ring of 3 buffers ran as fast as 4,
-// one of 2 about 13% slower; the FP16 kernel (no lo weights) with 3 buffers
-// fits the 164 KiB configuration, whose 92 KiB of L1 made it 3% faster than
-// with 4. So: 3 buffers when they stay within the 196 KiB configuration,
-// else the largest ring that fits at all.
+// fused kernel from 2.79 to 3.93 ms. A ring of 3 buffers ran as fast as 4;
+// one of 2 takes a third longer (4.19M torus camera rays 2.18 and 2.87 ms: a
+// buffer is refilled only once the next chunk is full and its shared points are
+// copied out); the FP16 kernel (no lo weights) with 3 buffers fits the 164 KiB
+// configuration, whose 92 KiB of L1 made it 3% faster than with 4. So: 3
+// buffers when they stay within the 196 KiB configuration, else the largest
+// ring that fits at all.
 constexpr uint32_t kSmemL1Friendly = 195u * 1024u;
 
 static int pick_nbuf(const DevObject &h, int list_chunks, bool fp16) {

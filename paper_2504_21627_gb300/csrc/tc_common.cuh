@@ -152,8 +152,7 @@ __device__ __forceinline__ uint32_t core_off(int r, int kg, uint32_t sbo) {
 
 struct TileInfo {
   int32_t kmax, slot, stop;
-  int16_t rows;   // rows of the tile
-  int16_t loads;  // weight loads up to this tile (low 15 bits)
+  int32_t loads;  // weight loads up to this tile (fused.cu)
 };
 
 __host__ __device__ inline uint32_t lay_take(uint32_t &off, uint32_t bytes, uint32_t align) {
