@@ -163,6 +163,12 @@ struct Ring {
   int n;
 };
 
+// A wait of a whole warp: its lanes go on, or give up after an abort, together
+// (what follows are warp-wide loads of tensor memory).
+__device__ __forceinline__ bool warp_wait(uint64_t *bar, uint32_t parity, volatile int *abort_flag) {
+  return __all_sync(0xffffffffu, mbar_wait(su32(bar), parity, abort_flag)) != 0;
+}
+
 // Loader: `copy(j, t, s, slot)` for the j-th segment of this CTA. Every copy has
 // landed when it returns, also after an abort.
 template <typename Copy>
@@ -272,7 +278,7 @@ __global__ void __launch_bounds__(kFwdThreads) layer0_kernel(const __grid_consta
       const int buf = tiles & 1, use = tiles >> 1;
       const bool any = a.k[t * kTileM] > 0;
       if (any) {
-        if (!mbar_wait(su32(&acc_full[buf]), (uint32_t)(use & 1), &s_abort)) break;
+        if (!warp_wait(&acc_full[buf], (uint32_t)(use & 1), &s_abort)) break;
         ++tiles;
         tc_after();
       }
@@ -450,7 +456,7 @@ __global__ void __launch_bounds__(kGradThreads) layer0_grad_kernel(const __grid_
       const int kmax = a.k[t * kTileM];
       if (kmax <= first) break;
       const int buf = tiles & 1, use = tiles >> 1;
-      if (use > 0 && !mbar_wait(su32(&y_empty[buf]), (uint32_t)((use - 1) & 1), &s_abort)) { ok = false; break; }
+      if (use > 0 && !warp_wait(&y_empty[buf], (uint32_t)((use - 1) & 1), &s_abort)) { ok = false; break; }
       seen = max(seen, (kmax - first + step - 1) / step);
       uint8_t *yb = sY + (size_t)buf * 2 * y_term;
 #pragma unroll 2
@@ -479,7 +485,7 @@ __global__ void __launch_bounds__(kGradThreads) layer0_grad_kernel(const __grid_
       fence_async_smem();
       mbar_arrive(su32(&y_full[buf]));
       if (tiles % kFlush == kFlush - 1) {
-        if (!mbar_wait(su32(&acc_full), (uint32_t)((tiles / kFlush) & 1), &s_abort)) { ok = false; break; }
+        if (!warp_wait(&acc_full, (uint32_t)((tiles / kFlush) & 1), &s_abort)) { ok = false; break; }
         tc_after();
         flush();
         mbar_arrive(su32(&acc_empty));
@@ -487,7 +493,7 @@ __global__ void __launch_bounds__(kGradThreads) layer0_grad_kernel(const __grid_
       ++tiles;
     }
     if (ok && seen > 0) {
-      if (mbar_wait(su32(&done), 0u, &s_abort)) {
+      if (warp_wait(&done, 0u, &s_abort)) {
         tc_after();
         flush();
       }
